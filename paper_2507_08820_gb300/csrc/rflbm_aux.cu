@@ -2,6 +2,7 @@
 // FP64 moments and global diagnostics, and the noise-source test kernels. Every kernel
 // that touches the populations is instantiated for the three storage formats.
 #include "rflbm_aux.h"
+#include "wide.cuh"
 
 namespace rflbm_dev {
 
@@ -15,29 +16,101 @@ __device__ __forceinline__ double psi(int c, double u) {
   return c == 0 ? (2.0 / 3.0 - u * u) : 0.5 * (1.0 / 3.0 + c * u + u * u);
 }
 
+// Population with the velocity of tile entry (a, b, c) = (c_x + 1, c_y + 1, c_z + 1).
+__host__ __device__ constexpr int pop_at(int a, int b, int c) {
+  for (int k = 0; k < kQ; ++k)
+    if (cx_of(k) == a - 1 && cy_of(k) == b - 1 && cz_of(k) == c - 1) return k;
+  return 0;
+}
+
 // ---------------------------------------------------------------- initial states
+// The rest populations w_i rho0 in the element type of an import or export, rounded once on
+// the host.
+template <class Tio>
+struct RestPops {
+  Tio f[kQ];
+};
+template <class Tio>
+static RestPops<Tio> rest_pops(float rho0) {
+  RestPops<Tio> r;
+  for (int i = 0; i < kQ; ++i) r.f[i] = (Tio)(weight_of(i) * (double)rho0);
+  return r;
+}
+
+// delta = psi(c, u) / w_c - 1 for c = -1, 0, +1: 3 u^2 -+ 3 u, -3 u^2 / 2.
+__device__ __forceinline__ void psi_excess(Pair32 u, Pair32 (&d)[3]) {
+  const Pair32 q = pmul(u, u);
+  const Pair32 q3 = pmul(Pair32{3.0f, 0.0f}, q), u3 = pmul(Pair32{3.0f, 0.0f}, u);
+  d[0] = padd(q3, Pair32{-u3.hi, -u3.lo});
+  d[1] = pmul(Pair32{-1.5f, 0.0f}, q);
+  d[2] = padd(q3, u3);
+}
+
+// g_i = r psi(c_x, u_x) psi(c_y, u_y) psi(c_z, u_z) - w_i rho0 of one site in FP64.
 template <int kStore>
-__global__ void k_init_field(Geometry g, float rho0, StoreScale ss, const double* __restrict__ rho,
+__device__ __noinline__ void init_site_fp64(const Geometry& g, uint32_t s, float rho0, const StoreScale& ss, double r,
+                                            double ux, double uy, double uz, typename Storage<kStore>::T* dst) {
+  using S = Storage<kStore>;
+  const Neighbours nb = neighbours(s, g);
+#pragma unroll
+  for (int i = 0; i < kQ; ++i) {
+    const double f = r * psi(cx_of(i), ux) * psi(cy_of(i), uy) * psi(cz_of(i), uz);
+    dst[pop_slot(g, nb, s, i)] = S::store((float)(f - weight_of(i) * (double)rho0), class_of(i), ss);
+  }
+}
+
+// The same for every site, scattered to the view's slots. With psi(c, u) = w_c (1 + delta_c),
+// g_i / w_i = Q_ab + (rho0 + Q_ab) delta_c where Q_ab = r D_ab + (r - rho0) and 1 + D_ab =
+// (1 + delta_a)(1 + delta_b): no difference of nearly equal numbers is left, so sums of two
+// float32 values carry it to 2^-43 of its terms, and FP64 differs from it by no more than its own
+// dozen roundings of f_i. Where every value within these errors rounds to one float32 value,
+// that is the FP64 result; a site with any population that they leave open is redone in FP64
+// (rest states and velocities near 1e-8, where g_i is lost in the roundings of f_i; one site in
+// thousands for flows). Bound by the 32 bytes read and 108 written per site (146 us at
+// 192^3): with 100 FP64 operations for every site 192^3 took 1254 us, so 435.
+template <int kStore>
+__global__ void __launch_bounds__(kAuxBlock) k_init_field(Geometry g, float rho0, StoreScale ss, const double* __restrict__ rho,
                              const double* __restrict__ u, typename Storage<kStore>::T* __restrict__ dst) {
   using S = Storage<kStore>;
   const int64_t s = (int64_t)blockIdx.x * kAuxBlock + threadIdx.x;
   if (s >= g.n) return;
   const double r = rho ? rho[s] : (double)rho0;
   const double ux = u ? u[s] : 0.0, uy = u ? u[g.n + s] : 0.0, uz = u ? u[2 * (int64_t)g.n + s] : 0.0;
-  // scatter f_i(x) to plane i at x - c_i
-  const Neighbours nb = neighbours(site_of(s), g);
+  const double dr = r - (double)rho0;
+  // (below 2^16 no product of r with the three delta_c overflows)
+  bool open = !(pair_range(r, 16) && pair_range(dr, 16) && pair_range(ux, 16) && pair_range(uy, 16) && pair_range(uz, 16));
+  if (!open) {
+    const Neighbours nb = neighbours(site_of(s), g);
+    const Pair32 R = pair_of(r), dR = pair_of(dr);
+    Pair32 dx[3], dy[3], dz[3];
+    psi_excess(pair_of(ux), dx);
+    psi_excess(pair_of(uy), dy);
+    psi_excess(pair_of(uz), dz);
+    const float own = fmaf(0x1p-43f, fabsf(dR.hi), 0x1p-48f * (fabsf(R.hi) + rho0));
 #pragma unroll
-  for (int i = 0; i < kQ; ++i) {
-    const double f = r * psi(cx_of(i), ux) * psi(cy_of(i), uy) * psi(cz_of(i), uz);
-    dst[pop_slot(g, nb, site_of(s), i)] = S::store((float)(f - weight_of(i) * (double)rho0), class_of(i), ss);
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        const float Aab = fmaf(fabsf(dx[a].hi), fabsf(dy[b].hi), fabsf(dx[a].hi) + fabsf(dy[b].hi));
+        const Pair32 D = padd(padd(dx[a], dy[b]), pmul(dx[a], dy[b]));
+        const Pair32 Q = padd(pmul(R, D), dR);
+        const Pair32 P = padd(Pair32{rho0, 0.0f}, Q);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          constexpr double w[4] = {w1d(1) * w1d(1) * w1d(1), w1d(1) * w1d(1) * w1d(0), w1d(1) * w1d(0) * w1d(0),
+                                   w1d(0) * w1d(0) * w1d(0)};
+          const int cls = class_at(a, b, c);
+          const Pair32 W{(float)w[cls], (float)(w[cls] - (double)(float)w[cls])};
+          const Pair32 v = pmul(W, padd(Q, pmul(P, dz[c])));
+          const float A = fmaf(fabsf(dz[c].hi), 1.0f + Aab, Aab);  // over |f_i / w_i r - 1| without cancellation
+          const float err = W.hi * fmaf(fabsf(R.hi) * A, 0x1.1p-43f, own);
+          const float lo = __fadd_rn(v.hi, __fsub_rn(v.lo, err));
+          open = open || !(lo == __fadd_rn(v.hi, __fadd_rn(v.lo, err)));
+          dst[pop_slot(g, nb, site_of(s), pop_at(a, b, c))] = S::store(lo, cls, ss);
+        }
+      }
   }
-}
-
-// Population with the velocity of tile entry (a, b, c) = (c_x + 1, c_y + 1, c_z + 1).
-__host__ __device__ constexpr int pop_at(int a, int b, int c) {
-  for (int k = 0; k < kQ; ++k)
-    if (cx_of(k) == a - 1 && cy_of(k) == b - 1 && cz_of(k) == c - 1) return k;
-  return 0;
+  if (open) init_site_fp64<kStore>(g, site_of(s), rho0, ss, r, ux, uy, uz, dst);
 }
 
 // Thermal initial state: every mode of every site an independent normal of variance
@@ -97,9 +170,11 @@ __global__ void k_init_thermal(Geometry g, float rho0, float kT, StoreScale ss, 
     }
 }
 
+// Import and export move 216 bytes per site (f32): with the rest populations formed by four FP64
+// products in every thread 128^3 float32 took 96 us in and 116 us out, with them given 65 us both.
 // Import of public-layout populations (double: exact shift in FP64; float: in FP32).
 template <class Tin, int kStore>
-__global__ void k_set_populations(Geometry g, float rho0, StoreScale ss, const Tin* __restrict__ f,
+__global__ void k_set_populations(Geometry g, RestPops<Tin> rest, StoreScale ss, const Tin* __restrict__ f,
                                   typename Storage<kStore>::T* __restrict__ dst) {
   using S = Storage<kStore>;
   const int64_t s = (int64_t)blockIdx.x * kAuxBlock + threadIdx.x;
@@ -107,13 +182,13 @@ __global__ void k_set_populations(Geometry g, float rho0, StoreScale ss, const T
   const Neighbours nb = neighbours(site_of(s), g);
 #pragma unroll
   for (int i = 0; i < kQ; ++i) {
-    const Tin v = f[i * (int64_t)g.n + s] - (Tin)(weight_of(i) * (double)rho0);
+    const Tin v = f[i * (int64_t)g.n + s] - rest.f[i];
     dst[pop_slot(g, nb, site_of(s), i)] = S::store((float)v, class_of(i), ss);
   }
 }
 
 template <class Tout, int kStore>
-__global__ void k_get_populations(Geometry g, float rho0, StoreScale ss,
+__global__ void k_get_populations(Geometry g, RestPops<Tout> rest, StoreScale ss,
                                   const typename Storage<kStore>::T* __restrict__ src, Tout* __restrict__ f) {
   using S = Storage<kStore>;
   const int64_t s = (int64_t)blockIdx.x * kAuxBlock + threadIdx.x;
@@ -122,7 +197,7 @@ __global__ void k_get_populations(Geometry g, float rho0, StoreScale ss,
 #pragma unroll
   for (int i = 0; i < kQ; ++i) {
     const float v = S::load(src[pop_slot(g, nb, site_of(s), i)], class_of(i), ss);
-    f[i * (int64_t)g.n + s] = (Tout)v + (Tout)(weight_of(i) * (double)rho0);
+    f[i * (int64_t)g.n + s] = (Tout)v + rest.f[i];
   }
 }
 
@@ -321,22 +396,22 @@ cudaError_t launch_init_field(const Geometry& g, float rho0, const StoreScale& s
 }
 cudaError_t launch_set_populations_f64(const Geometry& g, float rho0, const StoreScale& ss, int kind,
                                        const double* f, void* dst, cudaStream_t st) {
-  RFLBM_STORE_DISPATCH(kind, (k_set_populations<double, K><<<blocks_for(g.n), kAuxBlock, 0, st>>>(g, rho0, ss, f, (ST<K>*)dst)));
+  RFLBM_STORE_DISPATCH(kind, (k_set_populations<double, K><<<blocks_for(g.n), kAuxBlock, 0, st>>>(g, rest_pops<double>(rho0), ss, f, (ST<K>*)dst)));
   return cudaGetLastError();
 }
 cudaError_t launch_set_populations_f32(const Geometry& g, float rho0, const StoreScale& ss, int kind,
                                        const float* f, void* dst, cudaStream_t st) {
-  RFLBM_STORE_DISPATCH(kind, (k_set_populations<float, K><<<blocks_for(g.n), kAuxBlock, 0, st>>>(g, rho0, ss, f, (ST<K>*)dst)));
+  RFLBM_STORE_DISPATCH(kind, (k_set_populations<float, K><<<blocks_for(g.n), kAuxBlock, 0, st>>>(g, rest_pops<float>(rho0), ss, f, (ST<K>*)dst)));
   return cudaGetLastError();
 }
 cudaError_t launch_get_populations_f64(const Geometry& g, float rho0, const StoreScale& ss, int kind,
                                        const void* src, double* f, cudaStream_t st) {
-  RFLBM_STORE_DISPATCH(kind, (k_get_populations<double, K><<<blocks_for(g.n), kAuxBlock, 0, st>>>(g, rho0, ss, (const ST<K>*)src, f)));
+  RFLBM_STORE_DISPATCH(kind, (k_get_populations<double, K><<<blocks_for(g.n), kAuxBlock, 0, st>>>(g, rest_pops<double>(rho0), ss, (const ST<K>*)src, f)));
   return cudaGetLastError();
 }
 cudaError_t launch_get_populations_f32(const Geometry& g, float rho0, const StoreScale& ss, int kind,
                                        const void* src, float* f, cudaStream_t st) {
-  RFLBM_STORE_DISPATCH(kind, (k_get_populations<float, K><<<blocks_for(g.n), kAuxBlock, 0, st>>>(g, rho0, ss, (const ST<K>*)src, f)));
+  RFLBM_STORE_DISPATCH(kind, (k_get_populations<float, K><<<blocks_for(g.n), kAuxBlock, 0, st>>>(g, rest_pops<float>(rho0), ss, (const ST<K>*)src, f)));
   return cudaGetLastError();
 }
 cudaError_t launch_get_sites(const Geometry& g, float rho0, const StoreScale& ss, int kind,
