@@ -73,4 +73,89 @@ __device__ __forceinline__ double scaled_double(long long t, int k) {
   return __hiloint2double((int)((uint32_t)(bits >> 32) | sign), (int)(uint32_t)bits);
 }
 
+// 1 / x to FP64 accuracy for a normal x far from overflow: the approximation instruction and
+// two Newton steps (4 FP64 operations), and a / x from it, corrected once (3).
+__device__ __forceinline__ double reciprocal64(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  y = __fma_rn(y, __fma_rn(-x, y, 1.0), y);
+  return __fma_rn(y, __fma_rn(-x, y, 1.0), y);
+}
+__device__ __forceinline__ double divide64(double a, double x, double inv_x) {
+  const double q = __dmul_rn(a, inv_x);
+  return __fma_rn(__fma_rn(-x, q, a), inv_x, q);
+}
+
+// Sums over one axis of a 3x3x3 tile after another: drho = sum g, j = sum g c, the raw second
+// moments s = sum g c_a c_b (xx, yy, zz, xy, xz, yz).
+__device__ __forceinline__ void raw_sums(const float (&G)[3][3][3], float (&m)[10]) {
+  float X0[3][3], X1[3][3], X2[3][3];
+#pragma unroll
+  for (int b = 0; b < 3; ++b)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      X2[b][c] = __fadd_rn(G[2][b][c], G[0][b][c]);
+      X1[b][c] = __fsub_rn(G[2][b][c], G[0][b][c]);
+      X0[b][c] = __fadd_rn(X2[b][c], G[1][b][c]);
+    }
+  const auto sum3 = [](float a, float b, float c) { return __fadd_rn(__fadd_rn(a, b), c); };
+  float T00[3], T01[3], T02[3], T10[3], T11[3], T20[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    T02[c] = __fadd_rn(X0[2][c], X0[0][c]);
+    T01[c] = __fsub_rn(X0[2][c], X0[0][c]);
+    T00[c] = __fadd_rn(T02[c], X0[1][c]);
+    T11[c] = __fsub_rn(X1[2][c], X1[0][c]);
+    T10[c] = sum3(X1[2][c], X1[0][c], X1[1][c]);
+    T20[c] = sum3(X2[2][c], X2[0][c], X2[1][c]);
+  }
+  m[6] = __fadd_rn(T00[2], T00[0]);
+  m[0] = __fadd_rn(m[6], T00[1]);
+  m[1] = sum3(T10[0], T10[1], T10[2]);
+  m[2] = sum3(T01[0], T01[1], T01[2]);
+  m[3] = __fsub_rn(T00[2], T00[0]);
+  m[4] = sum3(T20[0], T20[1], T20[2]);
+  m[5] = sum3(T02[0], T02[1], T02[2]);
+  m[7] = sum3(T11[0], T11[1], T11[2]);
+  m[8] = __fsub_rn(T10[2], T10[0]);
+  m[9] = __fsub_rn(T01[2], T01[0]);
+}
+
+// The same sums as integers in units of 2^(e - 56), where e is the least exponent with every
+// |g| < 2^e: each g is split on the grids 2^(e - 18) and 2^(e - 37); the sums of either part
+// are exact in float32 (27 2^18 units at most), and so is the remainder's to 2^(e - 53). An FP64
+// accumulation of the 27 terms keeps 2^(e - 50) or so. E = e + 126 (the exponent field of the
+// largest |g|), 60 <= E <= 240. G is used up.
+__device__ __forceinline__ void fixed_sums(float (&G)[3][3][3], uint32_t E, long long (&t)[10]) {
+  const float half23 = 12582912.0f;  // 1.5 2^23: adding it leaves the integer in the low bits
+  float m[10];
+#pragma unroll
+  for (int part = 0; part < 3; ++part) {
+    const uint32_t down = part == 0 ? 271u : (part == 1 ? 290u : 309u);  // 1 / unit
+    if (part < 2) {
+      const float grid = __uint_as_float(((part == 0 ? E + 6u : E - 13u) << 23) | 0x400000u);
+      float H[3][3][3];
+#pragma unroll
+      for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int b = 0; b < 3; ++b)
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            H[a][b][c] = __fsub_rn(__fadd_rn(G[a][b][c], grid), grid);
+            G[a][b][c] = __fsub_rn(G[a][b][c], H[a][b][c]);
+          }
+      raw_sums(H, m);
+    } else {
+      raw_sums(G, m);
+    }
+    const float scale = __uint_as_float((down - E) << 23);
+#pragma unroll
+    for (int k = 0; k < 10; ++k) {
+      const int n = __float_as_int(__fmaf_rn(m[k], scale, half23)) - __float_as_int(half23);
+      if (part == 0) t[k] = n;
+      else t[k] = t[k] * 524288 + n;
+    }
+  }
+}
+
 }  // namespace rflbm_dev

@@ -45,3 +45,43 @@ def test_initial_fields_round_once(R, du, rho0, pattern):
     rest = o.weights()[:, None] * rho0
     scale = np.abs(rho) * np.prod([1.0 + 3 * np.abs(v) + 3 * v * v for v in u], axis=0) * o.weights()[:, None]
     assert np.all(np.abs(got - f) <= 2.0 ** -24 * np.abs(f - rest) + 256 * EPS * scale)
+
+
+def _state(shape, seed, scale):
+    g = np.random.default_rng(seed)
+    return scale * g.standard_normal((27, int(np.prod(shape)))) * 10.0 ** g.uniform(-6, 0, (27, int(np.prod(shape))))
+
+
+@pytest.mark.parametrize("scale", [0.0, 1e-28, 1e-16, 1e-3, 1e20, 1e36])
+@pytest.mark.parametrize("shape", [(1, 1, 1), (17, 9, 5), (256, 2, 1)])
+def test_moments_match_fp64_sums(R, scale, shape):
+    """rho0 = 1e-30 leaves g = f to one rounding, so that the sums of tiny and huge states are
+    compared at their own scale (outside 2^-66 .. 2^114 the kernel sums in FP64)."""
+    rho0 = 1e-30
+    f = _state(shape, 5, scale)
+    box = R.Box(*shape, tau=0.8, rho0=rho0)
+    R.rflbm_set_populations(box.h, np.ascontiguousarray(f))
+    f = box.populations()
+    rho, u, pi = box.macroscopic()
+    box.close()
+    wrho, wu, wpi = o.macroscopic(f)
+    s = np.abs(f).sum(axis=0) + 1e-30
+    assert np.all(np.abs(rho - wrho) <= 64 * EPS * s)
+    assert np.all(np.abs(pi - wpi) <= 64 * EPS * s)
+    ok = np.abs(wrho) > 1e-3 * s  # (a quotient by a density that cancels has no digits)
+    assert np.all(np.abs(u - wu)[:, ok] <= 1e-10 * (1.0 + np.abs(wu[:, ok])))
+
+
+def test_moments_of_non_finite_sites(R):
+    shape = (32, 3, 2)
+    f = o.rest_state(int(np.prod(shape)))
+    f[5, 17], f[0, 40] = np.nan, np.inf
+    box = R.Box(*shape, tau=0.8)
+    R.rflbm_set_populations(box.h, np.ascontiguousarray(f))
+    rho, u, pi = box.macroscopic()
+    st, status = R.rflbm_stats(box.h)
+    box.close()
+    assert np.isnan(rho[17]) and np.isinf(rho[40]) and np.all(np.isnan(u[:, 17]))
+    others = np.setdiff1d(np.arange(rho.size), [17, 40])
+    assert np.all(np.isfinite(rho[others])) and np.all(u[:, others] == 0.0)
+    assert status == R.RFLBM_EUNSTABLE and st.nonfinite == 2 and st.max_speed == 0.0
