@@ -449,6 +449,8 @@ rflbm_t* rflbm_create_ex(const rflbm_config_t* cfg) {
   h->stat_blocks = stats_partial_blocks(g, h->num_sms > 0 ? h->num_sms : 1);
   e = cudaMalloc((void**)&h->partials,
                  sizeof(double) * ((size_t)h->stat_blocks * kStatOutFields + 8));
+  if (e == cudaSuccess)
+    e = cudaMemset(h->partials + (size_t)h->stat_blocks * kStatOutFields, 0, 8 * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc((void**)&h->err, sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(h->err, 0, sizeof(int));
   if (e == cudaSuccess && h->slab) e = cudaEventCreateWithFlags(&h->faces_ready, cudaEventDisableTiming);

@@ -327,10 +327,8 @@ __global__ void __launch_bounds__(kAuxBlock) k_moments(Geometry g, double rho0, 
   }
 }
 
-// Per-block partial sums: drho, j (3), max |u|, count of unstable sites (non-finite, or
-// density not positive).
-constexpr int kStatFields = 6;
-
+// Partial sums: drho, j (3), max |u|, count of unstable sites (non-finite, or density not
+// positive).
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -342,54 +340,126 @@ __device__ __forceinline__ double warp_max(double v) {
   return v;
 }
 
-template <int kStore>
-__global__ void k_stats_partial(Geometry g, float rho0, StoreScale ss,
-                                const typename Storage<kStore>::T* __restrict__ src,
-                                double* __restrict__ partials) {
-  double acc[kStatFields] = {0, 0, 0, 0, 0, 0};
-  for (int64_t s = (int64_t)blockIdx.x * kAuxBlock + threadIdx.x; s < g.n;
-       s += (int64_t)gridDim.x * kAuxBlock) {
-    const SiteMoments m = site_moments<kStore, float>(g, site_of(s), src, ss);
-    const double r = (double)rho0 + m.drho;
-    // a non-finite site, or one whose density is not positive, counts as unstable
-    const bool stable = isfinite(m.drho) && isfinite(m.j[0]) && isfinite(m.j[1]) &&
-                        isfinite(m.j[2]) && r > 0.0;
-    if (stable) {
-      acc[0] += m.drho;
-      acc[1] += m.j[0]; acc[2] += m.j[1]; acc[3] += m.j[2];
-      const float sp = sqrtf((float)(m.j[0] * m.j[0] + m.j[1] * m.j[1] + m.j[2] * m.j[2])) / fabsf((float)r);
-      acc[4] = fmax(acc[4], (double)sp);
-    } else {
-      acc[5] += 1.0;
-    }
+// A running sum of float32 values as three of them: the rounding errors of each addition are
+// carried exactly into the next (the last one rounds), so that it holds more than the 53 bits
+// of an FP64 sum without an FP64 operation per term.
+struct RunningSum {
+  float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f;
+  __device__ __forceinline__ void add(float v) {
+    float e0, e1;
+    s0 = two_sum(s0, v, e0);
+    s1 = two_sum(s1, e0, e1);
+    s2 = __fadd_rn(s2, e1);
   }
-  __shared__ double sh[kAuxBlock / 32][kStatFields];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-  for (int f = 0; f < kStatFields; ++f) {
-    const double v = (f == 4) ? warp_max(acc[f]) : warp_sum(acc[f]);
-    if (lane == 0) sh[wid][f] = v;
-  }
-  __syncthreads();
-  if (threadIdx.x < kStatFields) {
-    const int f = threadIdx.x;
-    double v = sh[0][f];
-    for (int w = 1; w < kAuxBlock / 32; ++w) v = (f == 4) ? fmax(v, sh[w][f]) : v + sh[w][f];
-    partials[(int64_t)blockIdx.x * kStatFields + f] = v;
-  }
+  __device__ __forceinline__ double value() const { return ((double)s2 + (double)s1) + (double)s0; }
+};
+
+// x^2 + y^2 + z^2 rounded once from a sum with its rounding errors kept.
+__device__ __forceinline__ float sum_squares(float x, float y, float z) {
+  const float p = __fmul_rn(x, x), q = __fmul_rn(y, y), r = __fmul_rn(z, z);
+  float e1, e2;
+  const float s1 = two_sum(p, q, e1);
+  const float s2 = two_sum(s1, r, e2);
+  const float ep = __fmaf_rn(x, x, -p), eq = __fmaf_rn(y, y, -q), er = __fmaf_rn(z, z, -r);
+  return __fadd_rn(s2, __fadd_rn(__fadd_rn(e1, e2), __fadd_rn(ep, __fadd_rn(eq, er))));
 }
 
-// Fixed-order final reduction (one warp per field; deterministic for a fixed grid).
-__global__ void k_stats_final(const double* __restrict__ partials, int nblocks,
-                              double* __restrict__ out) {
-  const int f = blockIdx.x;
-  double v = 0.0;
-  for (int b = threadIdx.x; b < nblocks; b += 32) {
-    const double p = partials[(int64_t)b * kStatFields + f];
-    v = (f == 4) ? fmax(v, p) : v + p;
+__device__ __noinline__ float speed64(float x, float y, float z, float r) {
+  return (float)(sqrt((double)x * x + (double)y * y + (double)z * z) / (double)r);
+}
+
+// Global sums: every block sums the sites of its stride into one row of partials, and the last
+// block to finish adds the rows in a fixed order into out. Bound by the 108 bytes read per
+// site. A site's sums are taken into FP64 once per thread (RunningSum), not once per site: with
+// 20 FP64 operations per site, and the final sum in a launch of its own, 128^3 float32 took
+// 375 + 7 us, so 180.
+constexpr int kStatSums = 4;  // drho, j
+template <int kStore>
+__global__ void __launch_bounds__(kAuxBlock, 4) k_stats(Geometry g, float rho0, StoreScale ss,
+                                const typename Storage<kStore>::T* __restrict__ src,
+                                double* __restrict__ partials, double* __restrict__ out, unsigned* __restrict__ done) {
+  using S = Storage<kStore>;
+  RunningSum acc[kStatSums];
+  double big[kStatSums] = {0, 0, 0, 0};  // values of 2^100 and more
+  float vmax = 0.0f;
+  int bad = 0;
+#pragma unroll 1
+  for (int64_t s = (int64_t)blockIdx.x * kAuxBlock + threadIdx.x; s < g.n; s += (int64_t)gridDim.x * kAuxBlock) {
+    const Neighbours nb = neighbours(site_of(s), g);
+    float m[kStatSums] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+    for (int i = 0; i < kQ; ++i) {
+      const float v = S::load(src[pop_slot(g, nb, site_of(s), i)], class_of(i), ss);
+      m[0] += v;
+      if (cx_of(i)) m[1] += cx_of(i) * v;
+      if (cy_of(i)) m[2] += cy_of(i) * v;
+      if (cz_of(i)) m[3] += cz_of(i) * v;
+    }
+    const float r = __fadd_rn(rho0, m[0]);
+    const float mj = fmaxf(fabsf(m[1]), fmaxf(fabsf(m[2]), fabsf(m[3])));
+    // a non-finite site, or one whose density is not positive, counts as unstable
+    if (!(isfinite(m[0]) && isfinite(m[1]) && isfinite(m[2]) && isfinite(m[3]) && r > 0.0f)) {
+      ++bad;
+    } else if (fmaxf(fabsf(m[0]), mj) < 0x1p100f) {
+#pragma unroll
+      for (int f = 0; f < kStatSums; ++f) acc[f].add(m[f]);
+      // outside 2^-40 .. 2^60 the squares leave the range where their errors are exact
+      vmax = fmaxf(vmax, mj == 0.0f || (mj < 0x1p60f && mj > 0x1p-40f) ? sqrtf(sum_squares(m[1], m[2], m[3])) / r
+                                                                      : speed64(m[1], m[2], m[3], r));
+    } else {
+#pragma unroll
+      for (int f = 0; f < kStatSums; ++f) big[f] += (double)m[f];
+      vmax = fmaxf(vmax, speed64(m[1], m[2], m[3], r));
+    }
   }
-  v = (f == 4) ? warp_max(v) : warp_sum(v);
-  if (threadIdx.x == 0) out[f] = v;
+  // the block's row: warp f < 4 adds the threads' sums of field f, warp 4 their maxima and counts
+  __shared__ double sh[kStatSums][kAuxBlock];
+  __shared__ float shmax[kAuxBlock / 32];
+  __shared__ int shbad[kAuxBlock / 32];
+  __shared__ bool last;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+  for (int f = 0; f < kStatSums; ++f) sh[f][threadIdx.x] = acc[f].value() + big[f];
+  // (vmax >= 0: its bits order like integers)
+  const unsigned wmax = __reduce_max_sync(0xffffffffu, __float_as_uint(vmax));
+  const int wbad = __reduce_add_sync(0xffffffffu, bad);
+  if (lane == 0) {
+    shmax[wid] = __uint_as_float(wmax);
+    shbad[wid] = wbad;
+  }
+  __syncthreads();
+  double* const row = partials + (int64_t)blockIdx.x * kStatOutFields;
+  if (wid < kStatSums) {
+    double v = 0.0;
+    for (int k = lane; k < kAuxBlock; k += 32) v += sh[wid][k];
+    v = warp_sum(v);
+    if (lane == 0) row[wid] = v;
+  } else if (wid == kStatSums && lane == 0) {
+    float m = 0.0f;
+    int c = 0;
+    for (int w = 0; w < kAuxBlock / 32; ++w) {
+      m = fmaxf(m, shmax[w]);
+      c += shbad[w];
+    }
+    row[4] = (double)m;
+    row[5] = (double)c;
+  }
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(done, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  if (wid < kStatOutFields) {
+    double v = 0.0;
+    for (int b = lane; b < (int)gridDim.x; b += 32) {
+      const double p = __ldcg(partials + (int64_t)b * kStatOutFields + wid);
+      v = (wid == 4) ? fmax(v, p) : v + p;
+    }
+    v = (wid == 4) ? warp_max(v) : warp_sum(v);
+    if (lane == 0) out[wid] = v;
+  }
+  if (threadIdx.x == 0) *done = 0u;  // ready for the next call
 }
 
 // ---------------------------------------------------------------- noise tests
@@ -484,10 +554,10 @@ int stats_partial_blocks(const Geometry& g, int num_sms) {
   return (int)(want < cap ? (want > 0 ? want : 1) : cap);
 }
 cudaError_t launch_stats(const Geometry& g, float rho0, const StoreScale& ss, int kind,
-                         const void* src, double* partials, int nblocks, double* out6,
+                         const void* src, double* partials, int nblocks, double* out8,
                          cudaStream_t st) {
-  RFLBM_STORE_DISPATCH(kind, (k_stats_partial<K><<<nblocks, kAuxBlock, 0, st>>>(g, rho0, ss, (const ST<K>*)src, partials)));
-  k_stats_final<<<kStatFields, 32, 0, st>>>(partials, nblocks, out6);
+  unsigned* const done = reinterpret_cast<unsigned*>(out8 + kStatOutFields);
+  RFLBM_STORE_DISPATCH(kind, (k_stats<K><<<nblocks, kAuxBlock, 0, st>>>(g, rho0, ss, (const ST<K>*)src, partials, out8, done)));
   return cudaGetLastError();
 }
 cudaError_t launch_image_plane(const Geometry& g, size_t elem, const void* plane, int cx, int cy, int cz,

@@ -85,3 +85,25 @@ def test_moments_of_non_finite_sites(R):
     others = np.setdiff1d(np.arange(rho.size), [17, 40])
     assert np.all(np.isfinite(rho[others])) and np.all(u[:, others] == 0.0)
     assert status == R.RFLBM_EUNSTABLE and st.nonfinite == 2 and st.max_speed == 0.0
+
+
+@pytest.mark.parametrize("scale", [0.0, 1e-20, 1e-3, 1e18, 1e31, 1e36])
+@pytest.mark.parametrize("shape", [(1, 1, 1), (255, 1, 1), (257, 3, 1), (64, 48, 70)])
+def test_statistics_match_fp64_sums(R, scale, shape):
+    """Positive populations, so that every site is stable; values of 2^100 and more, and momenta
+    outside 2^-40 .. 2^60, take the FP64 branches. The sums of a site are float32."""
+    f = np.abs(_state(shape, 7, scale)) + o.weights()[:, None] * 1e-30
+    box = R.Box(*shape, tau=0.8, rho0=1e-30)
+    R.rflbm_set_populations(box.h, np.ascontiguousarray(f))
+    f = box.populations()
+    first, status = R.rflbm_stats(box.h)
+    st, _ = R.rflbm_stats(box.h)  # the count of finished blocks starts from zero again
+    box.close()
+    assert status == R.RFLBM_OK and st.nonfinite == 0
+    assert (first.mass, list(first.momentum), first.max_speed) == (st.mass, list(st.momentum), st.max_speed)
+    rho, u, _ = o.macroscopic(f)
+    s = np.abs(f).sum()
+    assert abs(st.mass - rho.sum()) <= 27 * 2.0 ** -24 * s
+    assert np.all(np.abs(np.array(st.momentum) - (rho * u).sum(axis=1)) <= 27 * 2.0 ** -24 * s)
+    speed = np.sqrt((u * u).sum(axis=0)).max()
+    assert abs(st.max_speed - speed) <= 60 * 2.0 ** -24 * max(1.0, speed)
