@@ -340,20 +340,6 @@ __device__ __forceinline__ double warp_max(double v) {
   return v;
 }
 
-// A running sum of float32 values as three of them: the rounding errors of each addition are
-// carried exactly into the next (the last one rounds), so that it holds more than the 53 bits
-// of an FP64 sum without an FP64 operation per term.
-struct RunningSum {
-  float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f;
-  __device__ __forceinline__ void add(float v) {
-    float e0, e1;
-    s0 = two_sum(s0, v, e0);
-    s1 = two_sum(s1, e0, e1);
-    s2 = __fadd_rn(s2, e1);
-  }
-  __device__ __forceinline__ double value() const { return ((double)s2 + (double)s1) + (double)s0; }
-};
-
 // x^2 + y^2 + z^2 rounded once from a sum with its rounding errors kept.
 __device__ __forceinline__ float sum_squares(float x, float y, float z) {
   const float p = __fmul_rn(x, x), q = __fmul_rn(y, y), r = __fmul_rn(z, z);

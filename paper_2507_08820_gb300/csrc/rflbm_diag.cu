@@ -4,6 +4,7 @@
 #include <cufft.h>
 
 #include "rflbm_diag.h"
+#include "wide.cuh"
 
 namespace rflbm_dev {
 
@@ -55,15 +56,20 @@ __device__ __forceinline__ void gather_tile(const typename Storage<kStore>::T* _
 }
 
 // Each thread accumulates up to kDiagSitesPerThread sites in float32, then the block sums
-// its 54 values in FP64 into one partial slot.
+// its 54 values into one FP64 partial slot: eight threads per column, each adding 32 of the
+// block's 256 values as a RunningSum, so that a column takes 40 FP64 operations per block.
+// (Warp shuffles in FP64 took 270 lane operations per value of a block and bound the kernel:
+// 128^3 float32 170 us.) Bound by the 108 bytes read per site.
+constexpr int kModePitch = kDiagBlock + 8;  // columns of a warp's four groups of eight in distinct banks
 template <int kStore>
-__global__ void __launch_bounds__(kDiagBlock) k_mode_sums(Geometry g, StoreScale ss,
+__global__ void __launch_bounds__(kDiagBlock, 2) k_mode_sums(Geometry g, StoreScale ss,
                                                           const typename Storage<kStore>::T* __restrict__ src,
                                                           double* __restrict__ partials) {
   float acc[2 * kQ];
 #pragma unroll
   for (int k = 0; k < 2 * kQ; ++k) acc[k] = 0.0f;
   const int64_t base = (int64_t)blockIdx.x * kDiagBlock * kDiagSitesPerThread;
+#pragma unroll 1
   for (int j = 0; j < kDiagSitesPerThread; ++j) {
     const int64_t s = base + (int64_t)j * kDiagBlock + threadIdx.x;
     if (s >= g.n) break;
@@ -81,32 +87,52 @@ __global__ void __launch_bounds__(kDiagBlock) k_mode_sums(Geometry g, StoreScale
           acc[kQ + k] = fmaf(M[p][q][r], M[p][q][r], acc[kQ + k]);
         }
   }
-  __shared__ double sh[kDiagBlock / 32][2 * kQ];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  __shared__ float sh[kQ][kModePitch];
 #pragma unroll
-  for (int k = 0; k < 2 * kQ; ++k) {
-    double v = (double)acc[k];
+  for (int half = 0; half < 2; ++half) {
+    if (half) __syncthreads();
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) sh[wid][k] = v;
-  }
-  __syncthreads();
-  if (threadIdx.x < 2 * kQ) {
+    for (int k = 0; k < kQ; ++k) sh[k][threadIdx.x] = acc[half * kQ + k];
+    __syncthreads();
+    const int col = threadIdx.x >> 3, part = threadIdx.x & 7;
     double v = 0.0;
-    for (int w = 0; w < kDiagBlock / 32; ++w) v += sh[w][threadIdx.x];
-    partials[(int64_t)blockIdx.x * 2 * kQ + threadIdx.x] = v;
+    if (col < kQ) {
+      RunningSum r;
+      bool big = false;
+#pragma unroll 8
+      for (int j = 0; j < kDiagBlock / 8; ++j) {
+        const float x = sh[col][part + 8 * j];
+        r.add(x);
+        big = big || !(fabsf(x) < 0x1p100f);
+      }
+      v = r.value();
+      if (big) {  // infinities, NaN and sums that could overflow float32
+        v = 0.0;
+        for (int j = 0; j < kDiagBlock / 8; ++j) v += (double)sh[col][part + 8 * j];
+      }
+    }
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (col < kQ && part == 0) partials[(int64_t)blockIdx.x * 2 * kQ + half * kQ + col] = v;
   }
 }
 
-__global__ void k_reduce_columns(const double* __restrict__ partials, int64_t rows, int cols,
+// Column sums of a row-major array in a fixed order: a block per column, thread t adds rows
+// t, t + 256, ..., then a fixed tree.
+__global__ void __launch_bounds__(kDiagBlock) k_reduce_columns(const double* __restrict__ partials, int64_t rows, int cols,
                                  double* __restrict__ out) {
-  // one warp per column, fixed order: lane l sums rows l, l + 32, ..., then a fixed tree
+  __shared__ double sh[kDiagBlock / 32];
   const int col = blockIdx.x;
   double v = 0.0;
-  for (int64_t r = threadIdx.x; r < rows; r += 32) v += partials[r * cols + col];
+  for (int64_t r = threadIdx.x; r < rows; r += kDiagBlock) v += partials[r * cols + col];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if (threadIdx.x == 0) out[col] = v;
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < kDiagBlock / 32; ++w) v += sh[w];
+    out[col] = v;
+  }
 }
 
 // Field value of one site, FP64 output from float32 sums of the shifted populations:
@@ -212,7 +238,7 @@ cudaError_t launch_mode_sums(const Geometry& g, const StoreScale& ss, int kind, 
     case kStoreBF16: k_mode_sums<kStoreBF16><<<(unsigned)blocks, kDiagBlock, 0, st>>>(g, ss, (const DT<kStoreBF16>*)src, partials); break;
     default: return cudaErrorInvalidValue;
   }
-  k_reduce_columns<<<2 * kQ, 32, 0, st>>>(partials, blocks, 2 * kQ, out54);
+  k_reduce_columns<<<2 * kQ, kDiagBlock, 0, st>>>(partials, blocks, 2 * kQ, out54);
   return cudaGetLastError();
 }
 
@@ -237,7 +263,7 @@ cudaError_t launch_shell_bins(const Geometry& g, const void* spec, int nshell, i
     if (e != cudaSuccess) return e;
   }
   k_shell_bins<<<blocks, kDiagBlock, smem, st>>>(g, (const cufftDoubleComplex*)spec, nshell, partials);
-  k_reduce_columns<<<2 * nshell, 32, 0, st>>>(partials, blocks, 2 * nshell, out);
+  k_reduce_columns<<<2 * nshell, kDiagBlock, 0, st>>>(partials, blocks, 2 * nshell, out);
   return cudaGetLastError();
 }
 

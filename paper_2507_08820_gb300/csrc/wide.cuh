@@ -86,6 +86,20 @@ __device__ __forceinline__ double divide64(double a, double x, double inv_x) {
   return __fma_rn(__fma_rn(-x, q, a), inv_x, q);
 }
 
+// A running sum of float32 values as three of them: the rounding errors of each addition are
+// carried exactly into the next (the last one rounds), so that it holds more than the 53 bits
+// of an FP64 sum without an FP64 operation per term.
+struct RunningSum {
+  float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f;
+  __device__ __forceinline__ void add(float v) {
+    float e0, e1;
+    s0 = two_sum(s0, v, e0);
+    s1 = two_sum(s1, e0, e1);
+    s2 = __fadd_rn(s2, e1);
+  }
+  __device__ __forceinline__ double value() const { return ((double)s2 + (double)s1) + (double)s0; }
+};
+
 // Sums over one axis of a 3x3x3 tile after another: drho = sum g, j = sum g c, the raw second
 // moments s = sum g c_a c_b (xx, yy, zz, xy, xz, yz).
 __device__ __forceinline__ void raw_sums(const float (&G)[3][3][3], float (&m)[10]) {

@@ -107,3 +107,18 @@ def test_statistics_match_fp64_sums(R, scale, shape):
     assert np.all(np.abs(np.array(st.momentum) - (rho * u).sum(axis=1)) <= 27 * 2.0 ** -24 * s)
     speed = np.sqrt((u * u).sum(axis=0)).max()
     assert abs(st.max_speed - speed) <= 60 * 2.0 ** -24 * max(1.0, speed)
+
+
+@pytest.mark.parametrize("n", [1, 31, 4095, 4096, 4097, 9001])
+def test_mode_sums_at_block_edges(R, n):
+    f = o.rest_state(n) + W.population_perturbation(n, 9, 1e-3)
+    box = R.Box(n, 1, 1, tau=0.8)
+    R.rflbm_set_populations(box.h, np.ascontiguousarray(f))
+    m = o.moments(box.populations())
+    m[0] -= 1.0
+    s1, s2 = R.rflbm_mode_sums(box.h)
+    box.close()
+    # per-site values to 27 float32 roundings of at most sum |g|, then sums of 16 sites in float32
+    tol = 64 * 2.0 ** -24 * np.abs(W.population_perturbation(n, 9, 1e-3)).sum(axis=0).max()
+    assert np.all(np.abs(s1 - m.sum(axis=1)) <= n * tol)
+    assert np.all(np.abs(s2 - (m * m).sum(axis=1)) <= n * tol * np.abs(m).max() * 4)
