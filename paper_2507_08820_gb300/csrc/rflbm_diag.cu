@@ -136,10 +136,13 @@ __global__ void __launch_bounds__(kDiagBlock) k_reduce_columns(const double* __r
 }
 
 // Field value of one site, FP64 output from float32 sums of the shifted populations:
-// 0 rho - rho0, 1..3 rho u, 4..9 Pi = a^(2) (xx, yy, zz, xy, xz, yz).
-template <int kStore>
-__global__ void k_field(Geometry g, StoreScale ss, const typename Storage<kStore>::T* __restrict__ src,
-                        int field, double* __restrict__ out) {
+// 0 rho - rho0, 1..3 rho u, 4..9 Pi = a^(2) (xx, yy, zz, xy, xz, yz). One instance per field,
+// its weights compiled in (selected per population at run time they took 92 us at 128^3
+// float32); bound by the 108 bytes read and 8 written per site.
+template <int kStore, int kField>
+__global__ void __launch_bounds__(kDiagBlock) k_field(Geometry g, StoreScale ss,
+                                                      const typename Storage<kStore>::T* __restrict__ src,
+                                                      double* __restrict__ out) {
   const int64_t s = (int64_t)blockIdx.x * kDiagBlock + threadIdx.x;
   if (s >= g.n) return;
   const Neighbours nb = neighbours((uint32_t)s, g);
@@ -147,77 +150,105 @@ __global__ void k_field(Geometry g, StoreScale ss, const typename Storage<kStore
 #pragma unroll
   for (int i = 0; i < kQ; ++i) {
     const float x = Storage<kStore>::load(src[pop_slot(g, nb, (uint32_t)s, i)], class_of(i), ss);
-    const int cx = cx_of(i), cy = cy_of(i), cz = cz_of(i);
-    float w;
-    switch (field) {
-      case 0: w = 1.0f; break;
-      case 1: w = (float)cx; break;
-      case 2: w = (float)cy; break;
-      case 3: w = (float)cz; break;
-      case 4: w = (float)(cx * cx); break;
-      case 5: w = (float)(cy * cy); break;
-      case 6: w = (float)(cz * cz); break;
-      case 7: w = (float)(cx * cy); break;
-      case 8: w = (float)(cx * cz); break;
-      default: w = (float)(cy * cz); break;
-    }
+    const int c[3] = {cx_of(i), cy_of(i), cz_of(i)};
+    const float w = kField == 0  ? 1.0f
+                    : kField < 4 ? (float)c[(kField - 1) % 3]
+                    : kField < 7 ? (float)(c[(kField - 4) % 3] * c[(kField - 4) % 3])
+                                 : (float)(c[kField == 9 ? 1 : 0] * c[kField == 7 ? 1 : 2]);
     v = fmaf(w, x, v);
     drho += x;
   }
   // Pi_aa = sum g c_a^2 - drho / 3 (the rest state drops out)
-  if (field >= 4 && field <= 6) v -= drho * (1.0f / 3.0f);
+  if (kField >= 4 && kField <= 6) v -= drho * (1.0f / 3.0f);
   out[s] = (double)v;
+}
+
+// Shell of a wave vector: round(L |k| / 2 pi) with L |k| / 2 pi = L sqrt(fx^2 + fy^2 + fz^2), k_a / L_a =
+// f_a, rounded as the FP64 expression does. The float32 value decides unless it lies within
+// its error (a few 2^-24 relative) of a boundary between shells.
+__device__ __forceinline__ int shell_of(int kx, int ky, int kz, const Geometry& g, double L) {
+  const float Lf = (float)L;
+  const float x = (float)kx * (Lf / (float)g.nx), y = (float)ky * (Lf / (float)g.ny), z = (float)kz * (Lf / (float)g.nz);
+  const float t = sqrtf(fmaf(x, x, fmaf(y, y, z * z)));
+  const float n = rintf(t);
+  if (fabsf(fabsf(t - n) - 0.5f) > fmaf(t, 2e-6f, 1e-6f)) return (int)n;
+  const double fx = (double)kx / g.nx, fy = (double)ky / g.ny, fz = (double)kz / g.nz;
+  return (int)llrint(L * sqrt(fx * fx + fy * fy + fz * fz));
 }
 
 // Shell sums of |F(k)|^2 / N over the half spectrum of a D2Z transform (kx = 0 .. nx/2),
 // each non-redundant vector counted twice. Shell n = round(|k| L / 2 pi) with
 // L = max(nx, ny, nz). The sums are reproducible bit for bit: each warp owns a row of
-// shell bins in shared memory and its lanes add to it one after another in lane order,
-// over a fixed assignment of spectrum entries to warps; the rows are then summed in warp
-// order into the block's partial row. (Counts are small integers, exact in any order.)
-__global__ void k_shell_bins(Geometry g, const cufftDoubleComplex* __restrict__ spec, int nshell,
-                             double* __restrict__ partials) {
-  extern __shared__ double bins[];  // [nwarps][nshell] sums, then [nshell] counts
-  const int nw = blockDim.x / 32, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int j = threadIdx.x; j < (nw + 1) * nshell; j += blockDim.x) bins[j] = 0.0;
+// shell bins in shared memory. Along a spectrum row (ky, kz) the shell grows with kx, so the
+// vectors of one shell are neighbours: a segmented scan over the warp's lanes adds them up
+// (a fixed tree), and the last lane of each run adds the run to its bin, one spectrum row after
+// another. The rows are then summed in warp order into the block's partial row. (Counts are
+// integers, exact in any order.) Nine FP64 operations per vector; with the shell computed in
+// FP64 (three quotients and a root) and the lanes adding to the bins one after another, 128^3
+// took 190 us.
+__global__ void __launch_bounds__(kDiagBlock) k_shell_bins(Geometry g, FastDiv div_nxh, FastDiv div_ny,
+                                                           const cufftDoubleComplex* __restrict__ spec, int nshell,
+                                                           double* __restrict__ partials) {
+  constexpr int kWarps = kDiagBlock / 32;
+  extern __shared__ double bins[];  // [kWarps][nshell] sums, then [nshell] counts
+  unsigned* const counts = reinterpret_cast<unsigned*>(bins + (size_t)kWarps * nshell);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  for (int j = threadIdx.x; j < kWarps * nshell; j += kDiagBlock) bins[j] = 0.0;
+  for (int j = threadIdx.x; j < nshell; j += kDiagBlock) counts[j] = 0u;
   __syncthreads();
   double* const mine = bins + (size_t)wid * nshell;
-  double* const counts = bins + (size_t)nw * nshell;
   const int nxh = g.nx / 2 + 1;
-  const int64_t total = (int64_t)g.nz * g.ny * nxh;
+  const int64_t total = (int64_t)g.nz * g.ny * nxh;  // at most n
   const double L = (double)max(g.nx, max(g.ny, g.nz));
   const double inv_n = 1.0 / (double)g.n;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t wbase = (int64_t)blockIdx.x * blockDim.x + 32 * wid; wbase < total; wbase += stride) {
+  const unsigned upto = 0xffffffffu >> (31 - lane);  // lanes 0 .. lane
+  const int64_t stride = (int64_t)gridDim.x * kDiagBlock;
+  for (int64_t wbase = (int64_t)blockIdx.x * kDiagBlock + 32 * wid; wbase < total; wbase += stride) {
     const int64_t idx = wbase + lane;  // warp-uniform trip count
     int shell = nshell;
-    double v = 0.0, w = 0.0;
+    uint32_t row = 0xffffffffu;
+    double v = 0.0;
+    bool self = false;
     if (idx < total) {
-      const int kx = (int)(idx % nxh);
-      const int ky = (int)((idx / nxh) % g.ny);
-      const int kz = (int)(idx / ((int64_t)nxh * g.ny));
-      const double fx = (double)kx / g.nx;
-      const double fy = (double)(ky <= (int)g.ny / 2 ? ky : ky - (int)g.ny) / g.ny;
-      const double fz = (double)(kz <= (int)g.nz / 2 ? kz : kz - (int)g.nz) / g.nz;
-      shell = (int)llrint(L * sqrt(fx * fx + fy * fy + fz * fz));
-      const bool self = (kx == 0) || ((g.nx % 2 == 0) && kx == (int)g.nx / 2);
-      w = self ? 1.0 : 2.0;
+      row = fastdiv((uint32_t)idx, div_nxh);
+      const int kx = (int)((uint32_t)idx - row * (uint32_t)nxh);
+      const int kz = (int)fastdiv(row, div_ny);
+      const int ky = (int)(row - (uint32_t)kz * g.ny);
+      shell = min(nshell, shell_of(kx, ky <= (int)g.ny / 2 ? ky : ky - (int)g.ny,
+                                   kz <= (int)g.nz / 2 ? kz : kz - (int)g.nz, g, L));
+      self = (kx == 0) || ((g.nx % 2 == 0) && kx == (int)g.nx / 2);
       const cufftDoubleComplex c = spec[idx];
-      v = w * (c.x * c.x + c.y * c.y) * inv_n;
+      v = fma(c.x, c.x, c.y * c.y) * (self ? inv_n : 2.0 * inv_n);
     }
-    const bool ok = shell < nshell;
-    if (ok) atomicAdd(&counts[shell], w);
-    for (int src = 0; src < 32; ++src) {
-      if (lane == src && ok) mine[shell] += v;
+    const int before = __shfl_up_sync(0xffffffffu, shell, 1);
+    const uint32_t row_before = __shfl_up_sync(0xffffffffu, row, 1);
+    const unsigned heads = __ballot_sync(0xffffffffu, lane == 0 || before != shell || row_before != row);
+    const unsigned selfs = __ballot_sync(0xffffffffu, self);
+    const int start = 31 - __clz(heads & upto);  // first lane of this lane's run
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const double t = __shfl_up_sync(0xffffffffu, v, o);
+      if (lane - o >= start) v += t;
+    }
+    const bool tail = (lane == 31 || ((heads >> (lane + 1)) & 1u)) && shell < nshell;
+    if (tail) {
+      const unsigned run = upto & ~((1u << start) - 1u);
+      atomicAdd(&counts[shell], 2u * (unsigned)__popc(run) - (unsigned)__popc(run & selfs));
+    }
+    // runs of one spectrum row are of different shells
+    const uint32_t first = __shfl_sync(0xffffffffu, row, 0);
+    const uint32_t end = min(fastdiv((uint32_t)min(wbase + 31, total - 1), div_nxh), first + 31u);
+    for (uint32_t r = first; r <= end; ++r) {
+      if (tail && row == r) mine[shell] += v;
       __syncwarp();
     }
   }
   __syncthreads();
-  for (int j = threadIdx.x; j < nshell; j += blockDim.x) {
+  for (int j = threadIdx.x; j < nshell; j += kDiagBlock) {
     double sum = 0.0;
-    for (int k = 0; k < nw; ++k) sum += bins[(size_t)k * nshell + j];
+    for (int k = 0; k < kWarps; ++k) sum += bins[(size_t)k * nshell + j];
     partials[(int64_t)blockIdx.x * 2 * nshell + j] = sum;
-    partials[(int64_t)blockIdx.x * 2 * nshell + nshell + j] = counts[j];
+    partials[(int64_t)blockIdx.x * 2 * nshell + nshell + j] = (double)counts[j];
   }
 }
 
@@ -242,16 +273,27 @@ cudaError_t launch_mode_sums(const Geometry& g, const StoreScale& ss, int kind, 
   return cudaGetLastError();
 }
 
+template <int kStore, int kField>
+static cudaError_t launch_field_at(const Geometry& g, const StoreScale& ss, const void* src, int field, double* out,
+                                   cudaStream_t st) {
+  if constexpr (kField > 9) {
+    return cudaErrorInvalidValue;
+  } else {
+    if (field != kField) return launch_field_at<kStore, kField + 1>(g, ss, src, field, out, st);
+    const unsigned blocks = (unsigned)(((int64_t)g.n + kDiagBlock - 1) / kDiagBlock);
+    k_field<kStore, kField><<<blocks, kDiagBlock, 0, st>>>(g, ss, (const DT<kStore>*)src, out);
+    return cudaGetLastError();
+  }
+}
+
 cudaError_t launch_field(const Geometry& g, const StoreScale& ss, int kind, const void* src,
                          int field, double* out, cudaStream_t st) {
-  const unsigned blocks = (unsigned)((g.n + kDiagBlock - 1) / kDiagBlock);
   switch (kind) {
-    case kStoreF32: k_field<kStoreF32><<<blocks, kDiagBlock, 0, st>>>(g, ss, (const DT<kStoreF32>*)src, field, out); break;
-    case kStoreF16: k_field<kStoreF16><<<blocks, kDiagBlock, 0, st>>>(g, ss, (const DT<kStoreF16>*)src, field, out); break;
-    case kStoreBF16: k_field<kStoreBF16><<<blocks, kDiagBlock, 0, st>>>(g, ss, (const DT<kStoreBF16>*)src, field, out); break;
+    case kStoreF32: return launch_field_at<kStoreF32, 0>(g, ss, src, field, out, st);
+    case kStoreF16: return launch_field_at<kStoreF16, 0>(g, ss, src, field, out, st);
+    case kStoreBF16: return launch_field_at<kStoreBF16, 0>(g, ss, src, field, out, st);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 cudaError_t launch_shell_bins(const Geometry& g, const void* spec, int nshell, int blocks,
@@ -262,7 +304,8 @@ cudaError_t launch_shell_bins(const Geometry& g, const void* spec, int nshell, i
     const cudaError_t e = cudaFuncSetAttribute(k_shell_bins, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  k_shell_bins<<<blocks, kDiagBlock, smem, st>>>(g, (const cufftDoubleComplex*)spec, nshell, partials);
+  k_shell_bins<<<blocks, kDiagBlock, smem, st>>>(g, make_fastdiv(g.nx / 2 + 1), make_fastdiv(g.ny),
+                                                 (const cufftDoubleComplex*)spec, nshell, partials);
   k_reduce_columns<<<2 * nshell, kDiagBlock, 0, st>>>(partials, blocks, 2 * nshell, out);
   return cudaGetLastError();
 }

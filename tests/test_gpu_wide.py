@@ -9,6 +9,7 @@ import pytest
 
 from oracle import rflbm_oracle as o
 from paper_2507_08820_gb300 import workloads as W
+from test_gpu_diag import _shells_numpy
 
 pytestmark = pytest.mark.gpu
 EPS = 2.0 ** -53
@@ -122,3 +123,21 @@ def test_mode_sums_at_block_edges(R, n):
     tol = 64 * 2.0 ** -24 * np.abs(W.population_perturbation(n, 9, 1e-3)).sum(axis=0).max()
     assert np.all(np.abs(s1 - m.sum(axis=1)) <= n * tol)
     assert np.all(np.abs(s2 - (m * m).sum(axis=1)) <= n * tol * np.abs(m).max() * 4)
+
+
+@pytest.mark.parametrize("shape", [(2, 3, 5), (33, 31, 7), (64, 3, 2), (7, 64, 9), (130, 4, 3), (3, 2, 100)])
+@pytest.mark.parametrize("nshell", [None, 3])
+def test_shell_sums_of_uneven_boxes(R, shape, nshell):
+    """Spectrum rows shorter and longer than a warp, and fewer shells than the box has."""
+    n = int(np.prod(shape))
+    f = o.rest_state(n) + W.population_perturbation(n, 11, 1e-3)
+    box = R.Box(*shape, tau=0.8)
+    R.rflbm_set_populations(box.h, np.ascontiguousarray(f))
+    r, u, pi = o.macroscopic(box.populations())
+    ns = R.rflbm_shell_count(box.h)
+    for k, phi in ((0, r - 1.0), (2, u[1] * r), (5, pi[1]), (9, pi[5])):
+        want_s, want_c = _shells_numpy(phi, shape, ns)
+        got_s, got_c = R.rflbm_structure_factor(box.h, k, nshell)
+        assert np.array_equal(got_c, want_c[:got_c.size]), k
+        assert np.allclose(got_s, want_s[:got_s.size], rtol=1e-5, atol=1e-6 * want_s.max()), k
+    box.close()
