@@ -51,11 +51,11 @@ template <int kStore>
 __device__ __noinline__ void init_site_fp64(const Geometry& g, uint32_t s, float rho0, const StoreScale& ss, double r,
                                             double ux, double uy, double uz, typename Storage<kStore>::T* dst) {
   using S = Storage<kStore>;
-  const Neighbours nb = neighbours(s, g);
+  const PopSlots slots(s, g);
 #pragma unroll
   for (int i = 0; i < kQ; ++i) {
     const double f = r * psi(cx_of(i), ux) * psi(cy_of(i), uy) * psi(cz_of(i), uz);
-    dst[pop_slot(g, nb, s, i)] = S::store((float)(f - weight_of(i) * (double)rho0), class_of(i), ss);
+    dst[slots(i)] = S::store((float)(f - weight_of(i) * (double)rho0), class_of(i), ss);
   }
 }
 
@@ -67,7 +67,7 @@ __device__ __noinline__ void init_site_fp64(const Geometry& g, uint32_t s, float
 // that is the FP64 result; a site with any population that they leave open is redone in FP64
 // (rest states and velocities near 1e-8, where g_i is lost in the roundings of f_i; one site in
 // thousands for flows). Bound by the 32 bytes read and 108 written per site (146 us at
-// 192^3): with 100 FP64 operations for every site 192^3 took 1254 us, so 435.
+// 192^3): with 100 FP64 operations for every site 192^3 took 1254 us, so 380.
 template <int kStore>
 __global__ void __launch_bounds__(kAuxBlock) k_init_field(Geometry g, float rho0, StoreScale ss, const double* __restrict__ rho,
                              const double* __restrict__ u, typename Storage<kStore>::T* __restrict__ dst) {
@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(kAuxBlock) k_init_field(Geometry g, float rho0
   // (below 2^16 no product of r with the three delta_c overflows)
   bool open = !(pair_range(r, 16) && pair_range(dr, 16) && pair_range(ux, 16) && pair_range(uy, 16) && pair_range(uz, 16));
   if (!open) {
-    const Neighbours nb = neighbours(site_of(s), g);
+    const PopSlots slots(site_of(s), g);
     const Pair32 R = pair_of(r), dR = pair_of(dr);
     Pair32 dx[3], dy[3], dz[3];
     psi_excess(pair_of(ux), dx);
@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(kAuxBlock) k_init_field(Geometry g, float rho0
           const float err = W.hi * fmaf(fabsf(R.hi) * A, 0x1.1p-43f, own);
           const float lo = __fadd_rn(v.hi, __fsub_rn(v.lo, err));
           open = open || !(lo == __fadd_rn(v.hi, __fadd_rn(v.lo, err)));
-          dst[pop_slot(g, nb, site_of(s), pop_at(a, b, c))] = S::store(lo, cls, ss);
+          dst[slots(pop_at(a, b, c))] = S::store(lo, cls, ss);
         }
       }
   }
@@ -155,7 +155,7 @@ __global__ void k_init_thermal(Geometry g, float rho0, float kT, StoreScale ss, 
 #pragma unroll
     for (int c = 0; c < 3; ++c)
       line_inverse(Z[p][0][c], Z[p][1][c], Z[p][2][c], Y[p][0][c], Y[p][1][c], Y[p][2][c]);
-  const Neighbours nb = neighbours(site_of(s), g);
+  const PopSlots slots(site_of(s), g);
 #pragma unroll
   for (int b = 0; b < 3; ++b)
 #pragma unroll
@@ -164,7 +164,7 @@ __global__ void k_init_thermal(Geometry g, float rho0, float kT, StoreScale ss, 
       line_inverse(Y[0][b][c], Y[1][b][c], Y[2][b][c], o[0], o[1], o[2]);
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
-        dst[pop_slot(g, nb, site_of(s), pop_at(a, b, c))] =
+        dst[slots(pop_at(a, b, c))] =
             S::store((float)(w1d(a) * w1d(b) * w1d(c)) * o[a], class_at(a, b, c), ss);
       }
     }
@@ -179,11 +179,11 @@ __global__ void k_set_populations(Geometry g, RestPops<Tin> rest, StoreScale ss,
   using S = Storage<kStore>;
   const int64_t s = (int64_t)blockIdx.x * kAuxBlock + threadIdx.x;
   if (s >= g.n) return;
-  const Neighbours nb = neighbours(site_of(s), g);
+  const PopSlots slots(site_of(s), g);
 #pragma unroll
   for (int i = 0; i < kQ; ++i) {
     const Tin v = f[i * (int64_t)g.n + s] - rest.f[i];
-    dst[pop_slot(g, nb, site_of(s), i)] = S::store((float)v, class_of(i), ss);
+    dst[slots(i)] = S::store((float)v, class_of(i), ss);
   }
 }
 
@@ -193,10 +193,10 @@ __global__ void k_get_populations(Geometry g, RestPops<Tout> rest, StoreScale ss
   using S = Storage<kStore>;
   const int64_t s = (int64_t)blockIdx.x * kAuxBlock + threadIdx.x;
   if (s >= g.n) return;
-  const Neighbours nb = neighbours(site_of(s), g);
+  const PopSlots slots(site_of(s), g);
 #pragma unroll
   for (int i = 0; i < kQ; ++i) {
-    const float v = S::load(src[pop_slot(g, nb, site_of(s), i)], class_of(i), ss);
+    const float v = S::load(src[slots(i)], class_of(i), ss);
     f[i * (int64_t)g.n + s] = (Tout)v + rest.f[i];
   }
 }
@@ -209,10 +209,10 @@ __global__ void k_get_sites(Geometry g, float rho0, StoreScale ss,
   const int64_t j = (int64_t)blockIdx.x * kAuxBlock + threadIdx.x;
   if (j >= n) return;
   const uint32_t s = site_of(sites[j]);
-  const Neighbours nb = neighbours(s, g);
+  const PopSlots slots(s, g);
 #pragma unroll
   for (int i = 0; i < kQ; ++i) {
-    f[i * n + j] = (double)S::load(src[pop_slot(g, nb, s, i)], class_of(i), ss) +
+    f[i * n + j] = (double)S::load(src[slots(i)], class_of(i), ss) +
                    weight_of(i) * (double)rho0;
   }
 }
@@ -228,12 +228,12 @@ template <int kStore, class Acc>
 __device__ __forceinline__ SiteMoments site_moments(const Geometry& g, uint32_t s,
                                                     const typename Storage<kStore>::T* src,
                                                     const StoreScale& ss) {
-  const Neighbours nb = neighbours(s, g);
+  const PopSlots slots(s, g);
   using S = Storage<kStore>;
   Acc drho = 0, j0 = 0, j1 = 0, j2 = 0, s0 = 0, s1 = 0, s2 = 0, s3 = 0, s4 = 0, s5 = 0;
 #pragma unroll
   for (int i = 0; i < kQ; ++i) {
-    const Acc v = (Acc)S::load(src[pop_slot(g, nb, s, i)], class_of(i), ss);
+    const Acc v = (Acc)S::load(src[slots(i)], class_of(i), ss);
     const int cx = cx_of(i), cy = cy_of(i), cz = cz_of(i);
     drho += v;
     if (cx) j0 += cx * v;
@@ -276,7 +276,7 @@ __device__ __noinline__ void moments_fp64(const Geometry& g, uint32_t s, const S
 // FP64 moments of every site: sums of 27 float32 values carried in 64-bit integers (fixed_sums),
 // packed into FP64 by integer operations, so that 15 FP64 operations per site are left (the
 // density and the three quotients) where plain FP64 takes 250. Bound by the 108 bytes read and
-// 80 written per site (196 us at 192^3; plain FP64 3224 us, so 389). Values outside the split's range (a population of 2^114 or more, or all
+// 80 written per site (196 us at 192^3; plain FP64 3224 us, so 337). Values outside the split's range (a population of 2^114 or more, or all
 // below 2^-66 and not zero; non-finite ones) go through FP64.
 template <int kStore>
 __global__ void __launch_bounds__(kAuxBlock) k_moments(Geometry g, double rho0, StoreScale ss,
@@ -288,10 +288,10 @@ __global__ void __launch_bounds__(kAuxBlock) k_moments(Geometry g, double rho0, 
   float G[3][3][3];
   uint32_t top = 0;
   {
-    const Neighbours nb = neighbours(site_of(s), g);
+    const PopSlots slots(site_of(s), g);
 #pragma unroll
     for (int i = 0; i < kQ; ++i) {
-      const float v = S::load(src[pop_slot(g, nb, site_of(s), i)], class_of(i), ss);
+      const float v = S::load(src[slots(i)], class_of(i), ss);
       G[cx_of(i) + 1][cy_of(i) + 1][cz_of(i) + 1] = v;
       top = max(top, __float_as_uint(v) & 0x7fffffffu);
     }
@@ -358,7 +358,7 @@ __device__ __noinline__ float speed64(float x, float y, float z, float r) {
 // block to finish adds the rows in a fixed order into out. Bound by the 108 bytes read per
 // site. A site's sums are taken into FP64 once per thread (RunningSum), not once per site: with
 // 20 FP64 operations per site, and the final sum in a launch of its own, 128^3 float32 took
-// 375 + 7 us, so 180.
+// 375 + 7 us, so 65.
 constexpr int kStatSums = 4;  // drho, j
 template <int kStore>
 __global__ void __launch_bounds__(kAuxBlock, 4) k_stats(Geometry g, float rho0, StoreScale ss,
@@ -371,11 +371,11 @@ __global__ void __launch_bounds__(kAuxBlock, 4) k_stats(Geometry g, float rho0, 
   int bad = 0;
 #pragma unroll 1
   for (int64_t s = (int64_t)blockIdx.x * kAuxBlock + threadIdx.x; s < g.n; s += (int64_t)gridDim.x * kAuxBlock) {
-    const Neighbours nb = neighbours(site_of(s), g);
+    const PopSlots slots(site_of(s), g);
     float m[kStatSums] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
     for (int i = 0; i < kQ; ++i) {
-      const float v = S::load(src[pop_slot(g, nb, site_of(s), i)], class_of(i), ss);
+      const float v = S::load(src[slots(i)], class_of(i), ss);
       m[0] += v;
       if (cx_of(i)) m[1] += cx_of(i) * v;
       if (cy_of(i)) m[2] += cy_of(i) * v;

@@ -48,11 +48,11 @@ template <int kStore>
 __device__ __forceinline__ void gather_tile(const typename Storage<kStore>::T* __restrict__ src,
                                             const Geometry& g, const StoreScale& ss, uint32_t s,
                                             float (&G)[3][3][3]) {
-  const Neighbours nb = neighbours(s, g);
+  const PopSlots slots(s, g);
 #pragma unroll
   for (int i = 0; i < kQ; ++i)
     G[cx_of(i) + 1][cy_of(i) + 1][cz_of(i) + 1] =
-        Storage<kStore>::load(src[pop_slot(g, nb, s, i)], class_of(i), ss);
+        Storage<kStore>::load(src[slots(i)], class_of(i), ss);
 }
 
 // Each thread accumulates up to kDiagSitesPerThread sites in float32, then the block sums
@@ -145,11 +145,11 @@ __global__ void __launch_bounds__(kDiagBlock) k_field(Geometry g, StoreScale ss,
                                                       double* __restrict__ out) {
   const int64_t s = (int64_t)blockIdx.x * kDiagBlock + threadIdx.x;
   if (s >= g.n) return;
-  const Neighbours nb = neighbours((uint32_t)s, g);
+  const PopSlots slots((uint32_t)s, g);
   float v = 0.0f, drho = 0.0f;
 #pragma unroll
   for (int i = 0; i < kQ; ++i) {
-    const float x = Storage<kStore>::load(src[pop_slot(g, nb, (uint32_t)s, i)], class_of(i), ss);
+    const float x = Storage<kStore>::load(src[slots(i)], class_of(i), ss);
     const int c[3] = {cx_of(i), cy_of(i), cz_of(i)};
     const float w = kField == 0  ? 1.0f
                     : kField < 4 ? (float)c[(kField - 1) % 3]

@@ -93,12 +93,30 @@ __device__ __forceinline__ uint32_t pull_site(const Neighbours& nb, int i) {
   return nb.X[cx_of(i) + 1] + nb.Y[cy_of(i) + 1] + nb.Z[cz_of(i) + 1];
 }
 
-// Element offset of g_i(s, t) in a buffer of view g.view (nb = neighbours(s, g)).
-__device__ __forceinline__ int64_t pop_slot(const Geometry& g, const Neighbours& nb, uint32_t s, int i) {
-  if (g.view == kViewNatural) return plane_of(i) * g.ps + s + g.zlo * g.nxy;
-  const int plane = g.view == kViewFlipped ? kQ - 1 - plane_of(i) : plane_of(i);
-  return plane * g.ps + pull_site(nb, i);
-}
+// Element offsets of the 27 values g_i(s, t) of site s in a buffer of view g.view. The view is
+// resolved once per site (the natural view has the site itself in place of its neighbours, the
+// flipped one counts the planes down from the last), so that the offsets are sums without
+// branches and a thread's 27 loads issue together (tested per population, the view kept the
+// statistics of 128^3 float32 at 180 us, so 65).
+struct PopSlots {
+  uint32_t X[3], YZ[3][3];
+  int64_t first, step;  // offset of plane 0, and from a plane to the next
+  __device__ __forceinline__ PopSlots(uint32_t s, const Geometry& g) {
+    const Neighbours nb = neighbours(s, g);
+    const bool own = g.view == kViewNatural;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      X[a] = own ? nb.X[1] : nb.X[a];
+#pragma unroll
+      for (int b = 0; b < 3; ++b) YZ[a][b] = own ? nb.Y[1] + nb.Z[1] : nb.Y[a] + nb.Z[b];
+    }
+    first = g.view == kViewFlipped ? (kQ - 1) * g.ps : 0;
+    step = g.view == kViewFlipped ? -g.ps : g.ps;
+  }
+  __device__ __forceinline__ int64_t operator()(int i) const {
+    return first + plane_of(i) * step + (X[cx_of(i) + 1] + YZ[cy_of(i) + 1][cz_of(i) + 1]);
+  }
+};
 
 // Signed offsets from site s to its periodic neighbours, per axis and per direction of
 // the pulled population: D?[a] is the offset of the coordinate minus (a - 1), so the
