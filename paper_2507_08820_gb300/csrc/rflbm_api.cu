@@ -19,6 +19,14 @@
 
 using namespace rflbm_dev;
 
+// Results of the synchronous calls, page-locked host memory: the kernels write it in place, so
+// that a call ends with one synchronisation and no copy.
+struct HostResults {
+  int err;
+  double stats[kStatOutFields];
+  double modes[2 * kQ];
+};
+
 struct rflbm {
   rflbm_config_t cfg;
   Geometry geo;
@@ -36,9 +44,10 @@ struct rflbm {
   bool initialised = false;
   StepVariant variant{};
   CollideParams cp{};
-  double* partials = nullptr;  // stats scratch: kStatOutFields doubles per block + 8 out
+  double* partials = nullptr;  // stats scratch: kStatOutFields doubles per block + the block count
   int stat_blocks = 0;
-  int* err = nullptr;          // device error flag set by bounded waits in kernels
+  HostResults* host = nullptr; // page-locked memory that kernels write the results of small calls into
+  int* err = nullptr;          // host->err: set by bounded waits in kernels
   int tma_width = 0;           // row-segment width of the TMA step path (0: generic)
   int kernel = RFLBM_KERNEL_GATHER;  // the step kernel in use
   CUtensorMap load_map[2];     // per buffer: source-row loads with halo
@@ -50,6 +59,8 @@ struct rflbm {
   double* diag_partials = nullptr;
   size_t diag_partials_bytes = 0;
   double* diag_field = nullptr;   // one FP64 field (N)
+  double* host_shells = nullptr;  // shell sums and counts (page-locked host memory)
+  int host_shells_n = 0;          // shells it holds
   void* diag_spec = nullptr;      // its D2Z spectrum
   cufftHandle fft_plan = 0;
   bool fft_ready = false;
@@ -241,10 +252,9 @@ int check_ready(const rflbm* h) {
 
 int sync(rflbm* h, const char* what) {
   RFLBM_CUDA(cudaStreamSynchronize(h->stream), what);
-  int flag = 0;
-  RFLBM_CUDA(cudaMemcpy(&flag, h->err, sizeof(int), cudaMemcpyDeviceToHost), "reading the error flag");
-  if (flag) {
-    cudaMemset(h->err, 0, sizeof(int));
+  volatile int* const flag = h->err;
+  if (*flag) {
+    *flag = 0;
     return fail(RFLBM_ETIMEOUT, "%s: a kernel gave up waiting for its bulk copies (bounded wait expired)", what);
   }
   return RFLBM_OK;
@@ -447,12 +457,14 @@ rflbm_t* rflbm_create_ex(const rflbm_config_t* cfg) {
     }
   }
   h->stat_blocks = stats_partial_blocks(g, h->num_sms > 0 ? h->num_sms : 1);
-  e = cudaMalloc((void**)&h->partials,
-                 sizeof(double) * ((size_t)h->stat_blocks * kStatOutFields + 8));
+  e = cudaMalloc((void**)&h->partials, sizeof(double) * ((size_t)h->stat_blocks * kStatOutFields + 1));
   if (e == cudaSuccess)
-    e = cudaMemset(h->partials + (size_t)h->stat_blocks * kStatOutFields, 0, 8 * sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc((void**)&h->err, sizeof(int));
-  if (e == cudaSuccess) e = cudaMemset(h->err, 0, sizeof(int));
+    e = cudaMemset(h->partials + (size_t)h->stat_blocks * kStatOutFields, 0, sizeof(double));
+  if (e == cudaSuccess) e = cudaHostAlloc((void**)&h->host, sizeof(HostResults), cudaHostAllocDefault);
+  if (e == cudaSuccess) {
+    std::memset(h->host, 0, sizeof(HostResults));
+    h->err = &h->host->err;
+  }
   if (e == cudaSuccess && h->slab) e = cudaEventCreateWithFlags(&h->faces_ready, cudaEventDisableTiming);
   if (e == cudaSuccess && h->slab) e = cudaEventCreateWithFlags(&h->exchanged, cudaEventDisableTiming);
   if (e != cudaSuccess) {
@@ -481,7 +493,8 @@ void rflbm_destroy(rflbm_t* h) {
     cudaFree(h->buf[1]);
   }
   cudaFree(h->partials);
-  cudaFree(h->err);
+  cudaFreeHost(h->host);
+  cudaFreeHost(h->host_shells);
   cudaFree(h->diag_partials);
   cudaFree(h->diag_field);
   cudaFree(h->diag_spec);
@@ -653,12 +666,11 @@ int rflbm_stats(rflbm_t* h, rflbm_stats_t* out) {
   if (int e = check_ready(h)) return e;
   if (!out) return fail(RFLBM_EINVAL, "stats output is NULL");
   DeviceGuard guard(h->device);
-  double* res = h->partials + (size_t)h->stat_blocks * kStatOutFields;
+  double* const host = h->host->stats;
+  unsigned* const done = reinterpret_cast<unsigned*>(h->partials + (size_t)h->stat_blocks * kStatOutFields);
   RFLBM_CUDA(launch_stats(vgeo(h), h->cp.rho0, h->ss, h->variant.storage, h->buf[h->cur], h->partials,
-                          h->stat_blocks, res, h->stream),
+                          h->stat_blocks, host, done, h->stream),
              "launching stats");
-  double host[kStatOutFields];
-  RFLBM_CUDA(cudaMemcpyAsync(host, res, sizeof(host), cudaMemcpyDeviceToHost, h->stream), "copying stats");
   if (int e = sync(h, "rflbm_stats")) return e;
   out->step = h->step;
   out->mass = (double)n_sites(h) * h->cfg.rho0 + host[0];
@@ -767,12 +779,10 @@ int rflbm_mode_sums(rflbm_t* h, double* sum, double* sumsq) {
   if (!sum || !sumsq) return fail(RFLBM_EINVAL, "outputs are NULL");
   DeviceGuard guard(h->device);
   const int64_t rows = mode_sum_blocks(h->geo);
-  if (int e = ensure_diag_partials(h, sizeof(double) * (size_t)(rows + 1) * 2 * kQ)) return e;
-  double* out = h->diag_partials + rows * 2 * kQ;
-  RFLBM_CUDA(launch_mode_sums(vgeo(h), h->ss, h->variant.storage, h->buf[h->cur], h->diag_partials, out, h->stream),
+  if (int e = ensure_diag_partials(h, sizeof(double) * (size_t)rows * 2 * kQ)) return e;
+  double* const host = h->host->modes;
+  RFLBM_CUDA(launch_mode_sums(vgeo(h), h->ss, h->variant.storage, h->buf[h->cur], h->diag_partials, host, h->stream),
              "launching mode sums");
-  double host[2 * kQ];
-  RFLBM_CUDA(cudaMemcpyAsync(host, out, sizeof(host), cudaMemcpyDeviceToHost, h->stream), "copying mode sums");
   if (int e = sync(h, "rflbm_mode_sums")) return e;
   for (int k = 0; k < kQ; ++k) {
     sum[k] = host[k];
@@ -805,17 +815,22 @@ int rflbm_structure_factor(rflbm_t* h, int field, int nshell, double* s_sum, dou
   }
   if (cufftSetStream(h->fft_plan, h->stream) != CUFFT_SUCCESS) return fail(RFLBM_ECUDA, "cufftSetStream failed");
   const int blocks = std::max(1, std::min(4 * std::max(h->num_sms, 1), (int)((nspec + 255) / 256)));
-  if (int e = ensure_diag_partials(h, sizeof(double) * (size_t)(blocks + 1) * 2 * nshell)) return e;
-  double* out = h->diag_partials + (size_t)blocks * 2 * nshell;
+  if (int e = ensure_diag_partials(h, sizeof(double) * (size_t)blocks * 2 * nshell)) return e;
+  if (h->host_shells_n < nshell) {
+    cudaFreeHost(h->host_shells);
+    h->host_shells = nullptr;
+    h->host_shells_n = 0;
+    RFLBM_CUDA(cudaHostAlloc((void**)&h->host_shells, sizeof(double) * 2 * (size_t)nshell, cudaHostAllocDefault),
+               "allocating the shell sums");
+    h->host_shells_n = nshell;
+  }
+  const double* const host = h->host_shells;
   RFLBM_CUDA(launch_field(vgeo(h), h->ss, h->variant.storage, h->buf[h->cur], field, h->diag_field, h->stream),
              "launching the field kernel");
   if (cufftExecD2Z(h->fft_plan, h->diag_field, (cufftDoubleComplex*)h->diag_spec) != CUFFT_SUCCESS)
     return fail(RFLBM_ECUDA, "cufftExecD2Z failed");
-  RFLBM_CUDA(launch_shell_bins(g, h->diag_spec, nshell, blocks, h->diag_partials, out, h->stream),
+  RFLBM_CUDA(launch_shell_bins(g, h->diag_spec, nshell, blocks, h->diag_partials, h->host_shells, h->stream),
              "launching the shell binning");
-  std::vector<double> host((size_t)2 * nshell);
-  RFLBM_CUDA(cudaMemcpyAsync(host.data(), out, sizeof(double) * host.size(), cudaMemcpyDeviceToHost, h->stream),
-             "copying the shell sums");
   if (int e = sync(h, "rflbm_structure_factor")) return e;
   for (int n = 0; n < nshell; ++n) {
     s_sum[n] = host[n];

@@ -540,10 +540,9 @@ int stats_partial_blocks(const Geometry& g, int num_sms) {
   return (int)(want < cap ? (want > 0 ? want : 1) : cap);
 }
 cudaError_t launch_stats(const Geometry& g, float rho0, const StoreScale& ss, int kind,
-                         const void* src, double* partials, int nblocks, double* out8,
+                         const void* src, double* partials, int nblocks, double* out, unsigned* done,
                          cudaStream_t st) {
-  unsigned* const done = reinterpret_cast<unsigned*>(out8 + kStatOutFields);
-  RFLBM_STORE_DISPATCH(kind, (k_stats<K><<<nblocks, kAuxBlock, 0, st>>>(g, rho0, ss, (const ST<K>*)src, partials, out8, done)));
+  RFLBM_STORE_DISPATCH(kind, (k_stats<K><<<nblocks, kAuxBlock, 0, st>>>(g, rho0, ss, (const ST<K>*)src, partials, out, done)));
   return cudaGetLastError();
 }
 cudaError_t launch_image_plane(const Geometry& g, size_t elem, const void* plane, int cx, int cy, int cz,

@@ -29,10 +29,10 @@ cudaError_t launch_moments(const Geometry& g, float rho0, const StoreScale& ss, 
 // Number of partial sums (blocks) the stats reduction uses for a box on a GPU with
 // num_sms multiprocessors; the scratch buffer holds kStatOutFields doubles per block.
 int stats_partial_blocks(const Geometry& g, int num_sms);
-// The sums go to out8[0..5]; out8[6] holds the count of finished blocks, zero before the first
-// call and after every one.
+// The sums go to out[0..5] (device memory or page-locked host memory); *done counts finished
+// blocks in device memory, zero before the first call and after every one.
 cudaError_t launch_stats(const Geometry& g, float rho0, const StoreScale& ss, int kind,
-                         const void* src, double* partials, int nblocks, double* out8,
+                         const void* src, double* partials, int nblocks, double* out, unsigned* done,
                          cudaStream_t st);
 // One plane of a state image (pull layout) from the plane of a population with velocity
 // (cx, cy, cz) held in the natural view; elem = 4 or 2 bytes per value.

@@ -516,9 +516,17 @@ struct rflbm_batch {
   int tile = 0;  // requested tile size (0: autotuned per row length, -1: by the order of preference)
   int ctas_per_sm = 1;
   unsigned long long* run = nullptr;  // device: first step of the current run, its buffer
-  int* err = nullptr;
+  // page-locked host memory that the kernels write in place: the results of the synchronous calls
+  struct HostResults {
+    int err;
+    double stats[kStatOutFields];
+  };
+  HostResults* results = nullptr;
+  int* err = nullptr;  // results->err
   double* partials = nullptr;
   int stat_blocks = 0;
+  void* staging = nullptr;  // exports of replicas, kept between calls (the largest so far)
+  size_t staging_bytes = 0;
   int64_t step = 0;
   bool initialised = false;
   cudaGraph_t graph = nullptr;
@@ -829,10 +837,9 @@ int enqueue_run(rflbm_batch* b, int64_t nsteps, cudaStream_t st) {
 
 int bsync(rflbm_batch* b, const char* what) {
   BCUDA(cudaStreamSynchronize(b->stream), what);
-  int flag = 0;
-  BCUDA(cudaMemcpy(&flag, b->err, sizeof(int), cudaMemcpyDeviceToHost), "reading the error flag");
-  if (flag) {
-    cudaMemset(b->err, 0, sizeof(int));
+  volatile int* const flag = b->err;
+  if (*flag) {
+    *flag = 0;
     return bfail(RFLBM_ETIMEOUT, "%s: a CTA gave up waiting for its bulk copies (bounded wait expired)", what);
   }
   return RFLBM_OK;
@@ -956,17 +963,20 @@ rflbm_batch_t* rflbm_batch_create(const rflbm_replica_t* reps, int n, double rho
   if (rc == RFLBM_OK) {
     cudaError_t e = cudaMalloc((void**)&b->run, 2 * sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaMemset(b->run, 0, 2 * sizeof(unsigned long long));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&b->err, sizeof(int));
-    if (e == cudaSuccess) e = cudaMemset(b->err, 0, sizeof(int));
+    if (e == cudaSuccess) e = cudaHostAlloc((void**)&b->results, sizeof(*b->results), cudaHostAllocDefault);
+    if (e == cudaSuccess) {
+      std::memset(b->results, 0, sizeof(*b->results));
+      b->err = &b->results->err;
+    }
     if (e != cudaSuccess) rc = bcuda(e, "allocating batch descriptors");
   }
   if (rc == RFLBM_OK) {
     int64_t nmax = 0;
     for (int r = 0; r < n; ++r) nmax = std::max<int64_t>(nmax, b->host[r].geo.n);
     b->stat_blocks = std::max(1, (int)std::min<int64_t>(4 * (int64_t)b->num_sms, (nmax + 255) / 256));
-    cudaError_t e = cudaMalloc((void**)&b->partials, sizeof(double) * ((size_t)b->stat_blocks * kStatOutFields + 8));
+    cudaError_t e = cudaMalloc((void**)&b->partials, sizeof(double) * ((size_t)b->stat_blocks * kStatOutFields + 1));
     if (e == cudaSuccess)
-      e = cudaMemset(b->partials + (size_t)b->stat_blocks * kStatOutFields, 0, 8 * sizeof(double));
+      e = cudaMemset(b->partials + (size_t)b->stat_blocks * kStatOutFields, 0, sizeof(double));
     if (e != cudaSuccess) rc = bcuda(e, "allocating the reduction scratch");
   }
   if (rc == RFLBM_OK) rc = layout_tiles(b, tile);
@@ -987,8 +997,9 @@ void rflbm_batch_destroy(rflbm_batch_t* b) {
   cudaFree(b->tile_rep);
   cudaFree(b->maps);
   cudaFree(b->run);
-  cudaFree(b->err);
+  cudaFreeHost(b->results);
   cudaFree(b->partials);
+  cudaFree(b->staging);
   if (b->exec) cudaGraphExecDestroy(b->exec);
   if (b->graph) cudaGraphDestroy(b->graph);
   for (cudaStream_t c : b->chains) cudaStreamDestroy(c);
@@ -1062,14 +1073,18 @@ int rflbm_batch_get_populations(rflbm_batch_t* b, int r, double* f) {
   if (!b || r < 0 || r >= b->n || !f) return bfail(RFLBM_EINVAL, "invalid batch, replica or output");
   if (!b->initialised) return bfail(RFLBM_ESTATE, "batch state not initialised");
   const ReplicaDev& d = b->host[r];
-  double* dev = nullptr;
   const size_t bytes = sizeof(double) * kQ * (size_t)d.geo.n;
-  BCUDA(cudaMalloc((void**)&dev, bytes), "allocating the export buffer");
-  cudaError_t e = launch_get_populations_f64(d.geo, d.cp.rho0, d.ss, b->storage, d.buf[b->cur], dev, b->stream);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(f, dev, bytes, cudaMemcpyDeviceToHost, b->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
-  cudaFree(dev);
-  if (e != cudaSuccess) return bcuda(e, "exporting replica populations");
+  if (b->staging_bytes < bytes) {
+    // (earlier exports are complete: every one ends with a synchronisation)
+    cudaFree(b->staging);
+    b->staging = nullptr;
+    b->staging_bytes = 0;
+    BCUDA(cudaMalloc(&b->staging, bytes), "allocating the export buffer");
+    b->staging_bytes = bytes;
+  }
+  BCUDA(launch_get_populations_f64(d.geo, d.cp.rho0, d.ss, b->storage, d.buf[b->cur], (double*)b->staging, b->stream),
+        "exporting replica populations");
+  BCUDA(cudaMemcpyAsync(f, b->staging, bytes, cudaMemcpyDeviceToHost, b->stream), "exporting replica populations");
   return bsync(b, "rflbm_batch_get_populations");
 }
 
@@ -1078,11 +1093,11 @@ int rflbm_batch_stats(rflbm_batch_t* b, int r, rflbm_stats_t* out) {
   if (!b->initialised) return bfail(RFLBM_ESTATE, "batch state not initialised");
   const ReplicaDev& d = b->host[r];
   const int blocks = std::max(1, (int)std::min<int64_t>(b->stat_blocks, ((int64_t)d.geo.n + 255) / 256));
-  double* res = b->partials + (size_t)b->stat_blocks * kStatOutFields;
-  BCUDA(launch_stats(d.geo, d.cp.rho0, d.ss, b->storage, d.buf[b->cur], b->partials, blocks, res, b->stream),
+  const double* const host = b->results->stats;
+  unsigned* const done = reinterpret_cast<unsigned*>(b->partials + (size_t)b->stat_blocks * kStatOutFields);
+  BCUDA(launch_stats(d.geo, d.cp.rho0, d.ss, b->storage, d.buf[b->cur], b->partials, blocks, b->results->stats, done,
+                     b->stream),
         "launching replica stats");
-  double host[kStatOutFields];
-  BCUDA(cudaMemcpyAsync(host, res, sizeof(host), cudaMemcpyDeviceToHost, b->stream), "copying replica stats");
   if (int e = bsync(b, "rflbm_batch_stats")) return e;
   out->step = b->step;
   out->mass = (double)d.geo.n * b->rho0 + host[0];
