@@ -16,6 +16,7 @@
 #include "../../include/rflbm_testing.h"
 #include "rflbm_aux.h"
 #include "rflbm_diag.h"
+#include "rflbm_spectrum.h"
 
 using namespace rflbm_dev;
 
@@ -58,11 +59,14 @@ struct rflbm {
   // diagnostics (allocated on first use)
   double* diag_partials = nullptr;
   size_t diag_partials_bytes = 0;
-  double* diag_field = nullptr;   // one FP64 field (N)
+  double* diag_field = nullptr;   // one field, then |F|^2 (8 N bytes)
   double* host_shells = nullptr;  // shell sums and counts (page-locked host memory)
   int host_shells_n = 0;          // shells it holds
-  void* diag_spec = nullptr;      // its D2Z spectrum
-  cufftHandle fft_plan = 0;
+  void* diag_spec = nullptr;      // its half spectrum
+  SpectrumAxis axes[3];           // the library's transform
+  float4* twiddles = nullptr;     // their tables
+  cufftHandle fft_plan = 0;       // cuFFT's, where an edge is none of the library's lengths
+  bool own_fft = false;
   bool fft_ready = false;
   void* staging = nullptr;     // device staging for host<->device transfers
   size_t staging_bytes = 0;
@@ -498,7 +502,8 @@ void rflbm_destroy(rflbm_t* h) {
   cudaFree(h->diag_partials);
   cudaFree(h->diag_field);
   cudaFree(h->diag_spec);
-  if (h->fft_ready) cufftDestroy(h->fft_plan);
+  if (h->fft_ready && !h->own_fft) cufftDestroy(h->fft_plan);
+  cudaFree(h->twiddles);
   cudaFree(h->staging);
   if (h->faces_ready) cudaEventDestroy(h->faces_ready);
   if (h->exchanged) cudaEventDestroy(h->exchanged);
@@ -807,13 +812,31 @@ int rflbm_structure_factor(rflbm_t* h, int field, int nshell, double* s_sum, dou
   const Geometry& g = h->geo;
   const size_t nspec = (size_t)g.nz * g.ny * (g.nx / 2 + 1);
   if (!h->fft_ready) {
-    RFLBM_CUDA(cudaMalloc((void**)&h->diag_field, sizeof(double) * g.n), "allocating the field buffer");
-    RFLBM_CUDA(cudaMalloc(&h->diag_spec, sizeof(cufftDoubleComplex) * nspec), "allocating the spectrum");
-    if (cufftPlan3d(&h->fft_plan, (int)g.nz, (int)g.ny, (int)g.nx, CUFFT_D2Z) != CUFFT_SUCCESS)
+    if (!h->diag_field)
+      RFLBM_CUDA(cudaMalloc((void**)&h->diag_field, sizeof(double) * g.n), "allocating the field buffer");
+    if (!h->diag_spec)
+      RFLBM_CUDA(cudaMalloc(&h->diag_spec, sizeof(cufftDoubleComplex) * nspec), "allocating the spectrum");
+    const int edge[3] = {(int)g.nx, (int)g.ny, (int)g.nz};
+    h->own_fft = true;
+    for (int a = 0; a < 3; ++a) h->own_fft = spectrum_axis(edge[a], &h->axes[a]) && h->own_fft;
+    if (h->own_fft) {
+      std::vector<float> table;
+      for (int a = 0; a < 3; ++a) {
+        const std::vector<float> t = spectrum_twiddles(edge[a]);
+        table.insert(table.end(), t.begin(), t.end());
+      }
+      if (!h->twiddles)
+        RFLBM_CUDA(cudaMalloc((void**)&h->twiddles, sizeof(float) * table.size()), "allocating the twiddle factors");
+      RFLBM_CUDA(cudaMemcpy(h->twiddles, table.data(), sizeof(float) * table.size(), cudaMemcpyHostToDevice),
+                 "copying the twiddle factors");
+      for (int a = 0, at = 0; a < 3; at += edge[a++]) h->axes[a].twiddles = h->twiddles + at;
+    } else if (cufftPlan3d(&h->fft_plan, edge[2], edge[1], edge[0], CUFFT_D2Z) != CUFFT_SUCCESS) {
       return fail(RFLBM_ECUDA, "cufftPlan3d failed for %u x %u x %u", g.nx, g.ny, g.nz);
+    }
     h->fft_ready = true;
   }
-  if (cufftSetStream(h->fft_plan, h->stream) != CUFFT_SUCCESS) return fail(RFLBM_ECUDA, "cufftSetStream failed");
+  if (!h->own_fft && cufftSetStream(h->fft_plan, h->stream) != CUFFT_SUCCESS)
+    return fail(RFLBM_ECUDA, "cufftSetStream failed");
   const int blocks = std::max(1, std::min(4 * std::max(h->num_sms, 1), (int)((nspec + 255) / 256)));
   if (int e = ensure_diag_partials(h, sizeof(double) * (size_t)blocks * 2 * nshell)) return e;
   if (h->host_shells_n < nshell) {
@@ -825,12 +848,23 @@ int rflbm_structure_factor(rflbm_t* h, int field, int nshell, double* s_sum, dou
     h->host_shells_n = nshell;
   }
   const double* const host = h->host_shells;
-  RFLBM_CUDA(launch_field(vgeo(h), h->ss, h->variant.storage, h->buf[h->cur], field, h->diag_field, h->stream),
-             "launching the field kernel");
-  if (cufftExecD2Z(h->fft_plan, h->diag_field, (cufftDoubleComplex*)h->diag_spec) != CUFFT_SUCCESS)
-    return fail(RFLBM_ECUDA, "cufftExecD2Z failed");
-  RFLBM_CUDA(launch_shell_bins(g, h->diag_spec, nshell, blocks, h->diag_partials, h->host_shells, h->stream),
-             "launching the shell binning");
+  const void* const src = h->buf[h->cur];
+  if (h->own_fft) {
+    float* const field_values = reinterpret_cast<float*>(h->diag_field);
+    RFLBM_CUDA(launch_field(vgeo(h), h->ss, h->variant.storage, src, field, field_values, h->stream),
+               "launching the field kernel");
+    RFLBM_CUDA(launch_power_spectrum(g, h->axes, field_values, h->diag_spec, h->diag_field, h->stream),
+               "launching the spectrum kernels");
+    RFLBM_CUDA(launch_power_bins(g, h->diag_field, nshell, blocks, h->diag_partials, h->host_shells, h->stream),
+               "launching the shell binning");
+  } else {
+    RFLBM_CUDA(launch_field(vgeo(h), h->ss, h->variant.storage, src, field, h->diag_field, h->stream),
+               "launching the field kernel");
+    if (cufftExecD2Z(h->fft_plan, h->diag_field, (cufftDoubleComplex*)h->diag_spec) != CUFFT_SUCCESS)
+      return fail(RFLBM_ECUDA, "cufftExecD2Z failed");
+    RFLBM_CUDA(launch_shell_bins(g, h->diag_spec, nshell, blocks, h->diag_partials, h->host_shells, h->stream),
+               "launching the shell binning");
+  }
   if (int e = sync(h, "rflbm_structure_factor")) return e;
   for (int n = 0; n < nshell; ++n) {
     s_sum[n] = host[n];

@@ -135,14 +135,15 @@ __global__ void __launch_bounds__(kDiagBlock) k_reduce_columns(const double* __r
   }
 }
 
-// Field value of one site, FP64 output from float32 sums of the shifted populations:
+// Field value of one site, float32 sums of the shifted populations (out in float32, or in FP64 for
+// cuFFT):
 // 0 rho - rho0, 1..3 rho u, 4..9 Pi = a^(2) (xx, yy, zz, xy, xz, yz). One instance per field,
 // its weights compiled in (selected per population at run time they took 92 us at 128^3
 // float32); bound by the 108 bytes read and 8 written per site.
-template <int kStore, int kField>
+template <int kStore, int kField, class Out>
 __global__ void __launch_bounds__(kDiagBlock) k_field(Geometry g, StoreScale ss,
                                                       const typename Storage<kStore>::T* __restrict__ src,
-                                                      double* __restrict__ out) {
+                                                      Out* __restrict__ out) {
   const int64_t s = (int64_t)blockIdx.x * kDiagBlock + threadIdx.x;
   if (s >= g.n) return;
   const PopSlots slots((uint32_t)s, g);
@@ -160,7 +161,7 @@ __global__ void __launch_bounds__(kDiagBlock) k_field(Geometry g, StoreScale ss,
   }
   // Pi_aa = sum g c_a^2 - drho / 3 (the rest state drops out)
   if (kField >= 4 && kField <= 6) v -= drho * (1.0f / 3.0f);
-  out[s] = (double)v;
+  out[s] = (Out)v;
 }
 
 // Shell of a wave vector: round(L |k| / 2 pi) with L |k| / 2 pi = L sqrt(fx^2 + fy^2 + fz^2), k_a / L_a =
@@ -176,7 +177,11 @@ __device__ __forceinline__ int shell_of(int kx, int ky, int kz, const Geometry& 
   return (int)llrint(L * sqrt(fx * fx + fy * fy + fz * fz));
 }
 
-// Shell sums of |F(k)|^2 / N over the half spectrum of a D2Z transform (kx = 0 .. nx/2),
+// |F|^2 of one entry of a spectrum: of its complex value, or given.
+__device__ __forceinline__ double power_of(const cufftDoubleComplex& c) { return fma(c.x, c.x, c.y * c.y); }
+__device__ __forceinline__ double power_of(double p) { return p; }
+
+// Shell sums of |F(k)|^2 / N over the half spectrum of a real transform (kx = 0 .. nx/2),
 // each non-redundant vector counted twice. Shell n = round(|k| L / 2 pi) with
 // L = max(nx, ny, nz). The sums are reproducible bit for bit: each warp owns a row of
 // shell bins in shared memory. Along a spectrum row (ky, kz) the shell grows with kx, so the
@@ -186,8 +191,9 @@ __device__ __forceinline__ int shell_of(int kx, int ky, int kz, const Geometry& 
 // integers, exact in any order.) Nine FP64 operations per vector; with the shell computed in
 // FP64 (three quotients and a root) and the lanes adding to the bins one after another, 128^3
 // took 190 us.
+template <class Entry>
 __global__ void __launch_bounds__(kDiagBlock) k_shell_bins(Geometry g, FastDiv div_nxh, FastDiv div_ny,
-                                                           const cufftDoubleComplex* __restrict__ spec, int nshell,
+                                                           const Entry* __restrict__ spec, int nshell,
                                                            double* __restrict__ partials) {
   constexpr int kWarps = kDiagBlock / 32;
   extern __shared__ double bins[];  // [kWarps][nshell] sums, then [nshell] counts
@@ -217,8 +223,7 @@ __global__ void __launch_bounds__(kDiagBlock) k_shell_bins(Geometry g, FastDiv d
       shell = min(nshell, shell_of(kx, ky <= (int)g.ny / 2 ? ky : ky - (int)g.ny,
                                    kz <= (int)g.nz / 2 ? kz : kz - (int)g.nz, g, L));
       self = (kx == 0) || ((g.nx % 2 == 0) && kx == (int)g.nx / 2);
-      const cufftDoubleComplex c = spec[idx];
-      v = fma(c.x, c.x, c.y * c.y) * (self ? inv_n : 2.0 * inv_n);
+      v = power_of(spec[idx]) * (self ? inv_n : 2.0 * inv_n);
     }
     const int before = __shfl_up_sync(0xffffffffu, shell, 1);
     const uint32_t row_before = __shfl_up_sync(0xffffffffu, row, 1);
@@ -273,8 +278,8 @@ cudaError_t launch_mode_sums(const Geometry& g, const StoreScale& ss, int kind, 
   return cudaGetLastError();
 }
 
-template <int kStore, int kField>
-static cudaError_t launch_field_at(const Geometry& g, const StoreScale& ss, const void* src, int field, double* out,
+template <int kStore, int kField, class Out>
+static cudaError_t launch_field_at(const Geometry& g, const StoreScale& ss, const void* src, int field, Out* out,
                                    cudaStream_t st) {
   if constexpr (kField > 9) {
     return cudaErrorInvalidValue;
@@ -286,8 +291,9 @@ static cudaError_t launch_field_at(const Geometry& g, const StoreScale& ss, cons
   }
 }
 
-cudaError_t launch_field(const Geometry& g, const StoreScale& ss, int kind, const void* src,
-                         int field, double* out, cudaStream_t st) {
+template <class Out>
+static cudaError_t launch_field_as(const Geometry& g, const StoreScale& ss, int kind, const void* src, int field, Out* out,
+                                   cudaStream_t st) {
   switch (kind) {
     case kStoreF32: return launch_field_at<kStoreF32, 0>(g, ss, src, field, out, st);
     case kStoreF16: return launch_field_at<kStoreF16, 0>(g, ss, src, field, out, st);
@@ -295,19 +301,36 @@ cudaError_t launch_field(const Geometry& g, const StoreScale& ss, int kind, cons
     default: return cudaErrorInvalidValue;
   }
 }
+cudaError_t launch_field(const Geometry& g, const StoreScale& ss, int kind, const void* src, int field, float* out,
+                         cudaStream_t st) {
+  return launch_field_as(g, ss, kind, src, field, out, st);
+}
+cudaError_t launch_field(const Geometry& g, const StoreScale& ss, int kind, const void* src, int field, double* out,
+                         cudaStream_t st) {
+  return launch_field_as(g, ss, kind, src, field, out, st);
+}
 
-cudaError_t launch_shell_bins(const Geometry& g, const void* spec, int nshell, int blocks,
-                              double* partials, double* out, cudaStream_t st) {
+template <class Entry>
+static cudaError_t launch_bins(const Geometry& g, const Entry* spec, int nshell, int blocks, double* partials, double* out,
+                               cudaStream_t st) {
   // kDiagBlock / 32 rows of sums + one row of counts: up to 221 KB at nshell = 3072
   const size_t smem = sizeof(double) * (size_t)(kDiagBlock / 32 + 1) * (size_t)nshell;
   if (smem > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(k_shell_bins, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e =
+        cudaFuncSetAttribute(k_shell_bins<Entry>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  k_shell_bins<<<blocks, kDiagBlock, smem, st>>>(g, make_fastdiv(g.nx / 2 + 1), make_fastdiv(g.ny),
-                                                 (const cufftDoubleComplex*)spec, nshell, partials);
+  k_shell_bins<<<blocks, kDiagBlock, smem, st>>>(g, make_fastdiv(g.nx / 2 + 1), make_fastdiv(g.ny), spec, nshell, partials);
   k_reduce_columns<<<2 * nshell, kDiagBlock, 0, st>>>(partials, blocks, 2 * nshell, out);
   return cudaGetLastError();
+}
+cudaError_t launch_shell_bins(const Geometry& g, const void* spec, int nshell, int blocks,
+                              double* partials, double* out, cudaStream_t st) {
+  return launch_bins(g, (const cufftDoubleComplex*)spec, nshell, blocks, partials, out, st);
+}
+cudaError_t launch_power_bins(const Geometry& g, const double* power, int nshell, int blocks, double* partials,
+                              double* out, cudaStream_t st) {
+  return launch_bins(g, power, nshell, blocks, partials, out, st);
 }
 
 }  // namespace rflbm_dev

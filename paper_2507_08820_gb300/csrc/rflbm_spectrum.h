@@ -1,0 +1,28 @@
+// The power spectrum of one field per site (rflbm_spectrum.cu).
+#pragma once
+
+#include <vector>
+
+#include "rflbm_internal.h"
+
+namespace rflbm_dev {
+
+// One axis of the transform: its length, the radices of its stages and its table of twiddle
+// factors exp(-2 pi i j / n) (device memory, n x (re hi, re lo, im hi, im lo)).
+struct SpectrumAxis {
+  int n, nfactors;
+  int factors[12];
+  int odd;   // 0: powers of two, 1: radices 3, 5 or 7 among them, 2: 11 or 13
+  const float4* twiddles;
+};
+
+// Fills *ax for length n (no table yet); false when n is above 768 or has a prime factor above 13.
+bool spectrum_axis(int n, SpectrumAxis* ax);
+std::vector<float> spectrum_twiddles(int n);
+
+// |F|^2 of the half spectrum, [kz][ky][kx], kx <= nx / 2, from the field (one float per site). spec
+// holds 16 bytes per value; power may be the field's memory.
+cudaError_t launch_power_spectrum(const Geometry& g, const SpectrumAxis (&ax)[3], const float* field, void* spec,
+                                  double* power, cudaStream_t st);
+
+}  // namespace rflbm_dev

@@ -125,10 +125,12 @@ def test_mode_sums_at_block_edges(R, n):
     assert np.all(np.abs(s2 - (m * m).sum(axis=1)) <= n * tol * np.abs(m).max() * 4)
 
 
-@pytest.mark.parametrize("shape", [(2, 3, 5), (33, 31, 7), (64, 3, 2), (7, 64, 9), (130, 4, 3), (3, 2, 100)])
+@pytest.mark.parametrize("shape", [(2, 3, 5), (33, 31, 7), (64, 3, 2), (7, 64, 9), (130, 4, 3), (3, 2, 100),
+                                   (768, 3, 1), (1, 5, 770), (11, 26, 8), (35, 9, 2), (1, 1, 6)])
 @pytest.mark.parametrize("nshell", [None, 3])
 def test_shell_sums_of_uneven_boxes(R, shape, nshell):
-    """Spectrum rows shorter and longer than a warp, and fewer shells than the box has."""
+    """Spectrum rows shorter and longer than a warp, fewer shells than the box has, every radix of
+    the library's transform, its longest edge, and edges it leaves to cuFFT (31, 770)."""
     n = int(np.prod(shape))
     f = o.rest_state(n) + W.population_perturbation(n, 11, 1e-3)
     box = R.Box(*shape, tau=0.8)
