@@ -126,7 +126,7 @@ def test_mode_sums_at_block_edges(R, n):
 
 
 @pytest.mark.parametrize("shape", [(2, 3, 5), (33, 31, 7), (64, 3, 2), (7, 64, 9), (130, 4, 3), (3, 2, 100),
-                                   (768, 3, 1), (1, 5, 770), (11, 26, 8), (35, 9, 2), (1, 1, 6)])
+                                   (768, 3, 1), (2, 5, 770), (11, 26, 8), (35, 9, 2), (1, 1, 6)])
 @pytest.mark.parametrize("nshell", [None, 3])
 def test_shell_sums_of_uneven_boxes(R, shape, nshell):
     """Spectrum rows shorter and longer than a warp, fewer shells than the box has, every radix of
