@@ -56,6 +56,7 @@ struct rflbm {
   CUtensorMap row_map;         // AA with one segment per row: three-plane row stores
   uint32_t test_extra_tx = 0;  // testing hook (rflbm_testing_expect_extra_bytes)
   bool has_row_map = false;
+  bool flat = false;           // the steps run in flat tiles (load_map, store_map are then flat)
   // diagnostics (allocated on first use)
   double* diag_partials = nullptr;
   size_t diag_partials_bytes = 0;
@@ -77,11 +78,6 @@ struct rflbm {
   cudaEvent_t exchanged = nullptr;    // recorded where the exchange ends
   cudaStream_t halo_stream = nullptr; // copies of rflbm_slab_exchange
 };
-
-namespace rflbm_dev {
-// The row-segment width for rows that no width divides (rflbm_step_tma.cu), 0 when none.
-int tma_ragged_width(uint32_t nx, size_t elem);
-}  // namespace rflbm_dev
 
 namespace {
 
@@ -270,6 +266,17 @@ bool encode_map(CUtensorMap* map, void* base, const Geometry& g, uint32_t box_x,
   return encode_population_map(map, base, g, box_x, 1, box_planes, storage);
 }
 
+// Flat tiles where they pay (whole boxes), when the descriptors encode.
+bool setup_flat(rflbm* h) {
+  const int st = h->variant.storage;
+  if (h->slab || h->cfg.kernel == RFLBM_KERNEL_GATHER || !flat_pays(h->geo, h->variant, h->aa)) return false;
+  for (int b = 0; b < (h->aa ? 1 : 2); ++b)
+    if (!encode_flat_map(&h->load_map[b], h->buf[b], h->geo, flat_load_sites(st), 3, st) ||
+        !encode_flat_map(&h->store_map[b], h->buf[b], h->geo, flat_store_sites(), kQ, st))
+      return false;
+  return true;
+}
+
 // Selects the TMA step path when the box allows it and the descriptors encode.
 void setup_tma(rflbm* h) {
   h->tma_width = 0;
@@ -278,6 +285,12 @@ void setup_tma(rflbm* h) {
   int w = tma_segment_width(h->geo.nx);
   // rows that no width divides: ragged last segments (whose excess threads store nothing)
   if (w == 0) w = tma_ragged_width(h->geo.nx, storage_bytes(st));
+  if (setup_flat(h)) {
+    h->flat = true;
+    h->tma_width = w;
+    h->kernel = w ? RFLBM_KERNEL_TMA : RFLBM_KERNEL_GATHER;
+    return;
+  }
   if (w == 0 || h->cfg.kernel == RFLBM_KERNEL_GATHER) return;
   const uint32_t halo = st == kStoreF32 ? 4 : 8;  // 16 bytes each side
   for (int b = 0; b < (h->aa ? 1 : 2); ++b) {
@@ -347,6 +360,21 @@ bool rflbm_dev::encode_population_map(CUtensorMap* map, void* base, const Geomet
                                                          : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
   return fn(map, dt, 4, base, dims, strides, box, estr,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+bool rflbm_dev::encode_flat_map(CUtensorMap* map, void* base, const Geometry& g, uint32_t box_sites,
+                                uint32_t box_planes, int storage) {
+  EncodeTiledFn fn = encode_tiled_fn();
+  if (!fn) return false;
+  const cuuint64_t dims[2] = {g.n, (cuuint64_t)kQ};
+  const cuuint64_t strides[1] = {(cuuint64_t)g.ps * storage_bytes(storage)};
+  const cuuint32_t box[2] = {box_sites, box_planes};
+  const cuuint32_t estr[2] = {1, 1};
+  const CUtensorMapDataType dt = storage == kStoreF16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
+                                 : storage == kStoreBF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16
+                                                         : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
+  return fn(map, dt, 2, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -587,6 +615,10 @@ cudaError_t launch_rows(rflbm* h, StepParams& p, uint32_t row0, uint32_t nrows, 
   if (h->aa) {
     p.src = p.dst = h->buf[0];
     const bool odd = h->phase != 0;
+    if (h->flat) {
+      const TmaMaps m{&h->load_map[0], &h->store_map[0], 0};
+      return launch_step_flat_aa(m, p, h->variant, odd, h->stream);
+    }
     if (h->tma_width) {
       const TmaMaps m{&h->load_map[0], &h->store_map[0], h->tma_width, h->has_row_map ? &h->row_map : nullptr};
       return launch_step_aa_tma(m, p, h->variant, odd, h->stream);
@@ -595,6 +627,10 @@ cudaError_t launch_rows(rflbm* h, StepParams& p, uint32_t row0, uint32_t nrows, 
   }
   p.src = h->buf[h->cur];
   p.dst = h->buf[1 - h->cur];
+  if (h->flat) {
+    const TmaMaps m{&h->load_map[h->cur], &h->store_map[1 - h->cur], 0};
+    return launch_step_flat(m, p, h->variant, h->stream);
+  }
   if (h->tma_width) {
     const TmaMaps m{&h->load_map[h->cur], &h->store_map[1 - h->cur], h->tma_width};
     return launch_step_tma(m, p, h->variant, h->stream);
@@ -989,7 +1025,9 @@ int rflbm_step_path(const rflbm_t* h, int* width) {
 
 int rflbm_step_sites_per_thread(const rflbm_t* h) {
   if (int e = check_handle(h)) return e;
-  if (h->kernel != RFLBM_KERNEL_TMA) return 1;
+  if (h->kernel != RFLBM_KERNEL_TMA && !h->flat) return 1;
+  if (h->flat)
+    return (h->aa ? flat_aa_uses_pairs(h->variant, h->phase != 0, h->geo.nx) : tma_uses_pairs(h->variant)) ? 2 : 1;
   if (h->aa) return aa_uses_pairs(h->variant, h->phase != 0, h->has_row_map) ? 2 : 1;
   return tma_uses_pairs(h->variant) ? 2 : 1;
 }

@@ -219,11 +219,32 @@ bool aa_uses_pairs(const StepVariant& v, bool odd, bool full_row);
 
 // Row-segment width of the TMA step kernels for a box of x edge nx (0: not supported).
 int tma_segment_width(uint32_t nx);
+// The width for rows that no width divides, with a ragged last segment (0: none).
+int tma_ragged_width(uint32_t nx, size_t elem);
 // Launches one step of a TMA-staged kernel on `stream` (any storage format).
 cudaError_t launch_step_tma(const TmaMaps& m, const StepParams& p, const StepVariant& v,
                             cudaStream_t stream);
 // The 16-bit storage part of launch_step_tma (rflbm_step_tma16.cu).
 cudaError_t launch_step_tma_16(const TmaMaps& m, const StepParams& p, const StepVariant& v,
                                cudaStream_t stream);
+
+// The flat-tile step kernels (step_flat.cuh), for whole boxes: whether a box runs in them, the
+// boxes of their tensor maps (m.load: flat_load_sites x 3 planes, m.store: flat_store_sites x 27
+// planes), and the launch of one step over all sites.
+bool flat_pays(const Geometry& g, const StepVariant& v, bool aa);
+// True when an AA step in flat tiles runs two sites per thread.
+bool flat_aa_uses_pairs(const StepVariant& v, bool odd, uint32_t nx);
+uint32_t flat_load_sites(int storage);
+uint32_t flat_store_sites();
+cudaError_t launch_step_flat(const TmaMaps& m, const StepParams& p, const StepVariant& v, cudaStream_t stream);
+cudaError_t launch_step_flat_16(const TmaMaps& m, const StepParams& p, const StepVariant& v, cudaStream_t stream);
+
+// One in-place AA step in flat tiles on the buffer p.dst (the even form loads and stores m.store).
+cudaError_t launch_step_flat_aa(const TmaMaps& m, const StepParams& p, const StepVariant& v, bool odd, cudaStream_t stream);
+
+// Encodes the buffer at `base` as a 2-D tensor (site, plane) of g.n sites for tiled copies of
+// (box_sites, box_planes) boxes; false if the driver refuses.
+bool encode_flat_map(CUtensorMap* map, void* base, const Geometry& g, uint32_t box_sites, uint32_t box_planes,
+                     int storage);
 
 }  // namespace rflbm_dev
