@@ -160,6 +160,17 @@ __device__ __forceinline__ void site_noise(uint32_t site, uint32_t step, uint32_
   site_noise_part<0, 6>(site, step, replica, k0, k1, out);
 }
 
+// True for every draw (no normal is a NaN). What a kernel does on this condition waits for the
+// first n normals: before griddepcontrol.wait it keeps the draw there, where the compiler would
+// otherwise move it behind the wait and the loads to hold fewer registers.
+template <int n>
+__device__ __forceinline__ bool normals_formed(const SiteNoise& noise) {
+  float sum = 0.0f;
+#pragma unroll
+  for (int m = 0; m < n; ++m) sum += noise.n[m];
+  return __float_as_uint(sum) != 0x7fc12345u;
+}
+
 // Normal n[m] (m = 0..23) of a SiteNoise.
 __device__ __forceinline__ float normal_at(const SiteNoise& n, int m) { return n.n[m]; }
 

@@ -56,6 +56,7 @@ struct rflbm {
   CUtensorMap row_map;         // AA with one segment per row: three-plane row stores
   uint32_t test_extra_tx = 0;  // testing hook (rflbm_testing_expect_extra_bytes)
   bool has_row_map = false;
+  bool small = false;          // the steps run in the general kernel for their latency
   bool flat = false;           // the steps run in flat tiles (load_map, store_map are then flat)
   // diagnostics (allocated on first use)
   double* diag_partials = nullptr;
@@ -277,11 +278,26 @@ bool setup_flat(rflbm* h) {
   return true;
 }
 
+// Whole boxes of the automatic choice whose TMA steps are slower than the general kernel's for
+// their latency alone. Microseconds per step, TMA against general: with noise 32^3 float32 6.5 and
+// 4.3, AA 5.3 and 2.9, float16 7.9 and 5.0; 96x32x32 5.6 and 4.7, float16 8.1 and 5.3;
+// 128x32x32 (131,072 sites) 6.3 and 6.6. Without noise float32 32^3 6.2 and 5.1, 96x32x32 6.1 and
+// 6.0; 16-bit 32^3 5.6 and 6.0.
+// Rows that no segment width divides: 56^3 (ragged segments) 9.2 and 8.5, without noise 9.6 and 6.3;
+// 80^3 without noise 17.9 and 15.8.
+bool general_pays(const rflbm* h) {
+  if (h->slab || h->cfg.kernel != RFLBM_KERNEL_AUTO) return false;
+  const bool noise = h->variant.noise, f32 = h->variant.storage == kStoreF32;
+  if (tma_segment_width(h->geo.nx) == 0) return h->geo.n < (noise ? 190000u : (f32 ? 450000u : 230000u));
+  return noise ? h->geo.n < 112000u : (f32 && h->geo.n < 60000u);
+}
+
 // Selects the TMA step path when the box allows it and the descriptors encode.
 void setup_tma(rflbm* h) {
   h->tma_width = 0;
   h->kernel = RFLBM_KERNEL_GATHER;
   const int st = h->variant.storage;
+  h->small = general_pays(h);
   int w = tma_segment_width(h->geo.nx);
   // rows that no width divides: ragged last segments (whose excess threads store nothing)
   if (w == 0) w = tma_ragged_width(h->geo.nx, storage_bytes(st));
@@ -612,9 +628,12 @@ cudaError_t launch_rows(rflbm* h, StepParams& p, uint32_t row0, uint32_t nrows, 
   p.nrows = nrows;
   p.row_split = split < nrows ? split : nrows;
   p.row_gap = gap;
+  // (the testing hook is about the TMA kernels' waits)
+  const bool general = h->small && !h->test_extra_tx;
   if (h->aa) {
     p.src = p.dst = h->buf[0];
     const bool odd = h->phase != 0;
+    if (general) return launch_step_aa_gather(p, h->variant, odd, h->stream);
     if (h->flat) {
       const TmaMaps m{&h->load_map[0], &h->store_map[0], 0};
       return launch_step_flat_aa(m, p, h->variant, odd, h->stream);
@@ -627,6 +646,7 @@ cudaError_t launch_rows(rflbm* h, StepParams& p, uint32_t row0, uint32_t nrows, 
   }
   p.src = h->buf[h->cur];
   p.dst = h->buf[1 - h->cur];
+  if (general) return launch_step_gather(p, h->variant, h->stream);
   if (h->flat) {
     const TmaMaps m{&h->load_map[h->cur], &h->store_map[1 - h->cur], 0};
     return launch_step_flat(m, p, h->variant, h->stream);

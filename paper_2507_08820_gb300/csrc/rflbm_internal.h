@@ -180,7 +180,7 @@ struct TmaMaps {
   const CUtensorMap* row3 = nullptr;  // AA, width == nx: box width x 1 x 1 x 3 planes
 };
 
-constexpr int kStepBlock = 256;
+constexpr int kStepBlock = 64;  // threads per block of the general kernel
 
 // Variant flags of the step kernel.
 struct StepVariant {

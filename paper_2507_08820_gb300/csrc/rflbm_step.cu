@@ -1,15 +1,22 @@
 // The fused stream-and-collide step (Eq. 25 / Eq. 12 followed by Eq. 8) in the pull
 // layout, for any box: the general kernel.
 //
-// One thread per site. The thread gathers the 27 pre-collision populations of its site
-// from the 27 neighbours x - c_i (periodic wrap; consecutive threads read consecutive
-// addresses of every plane, so each warp-wide load is one coalesced row segment), draws
-// its 24 normals (Philox4x32-10 + Box-Muller, independent of the loads so that the
-// arithmetic overlaps the memory latency), collides in registers and writes the 27
-// post-collision values to its own site of the other buffer (27 coalesced stores).
+// One thread per site. The thread draws its 24 normals (Philox4x32-10 + Box-Muller) while the
+// previous step drains (programmatic dependent launch), waits for it, gathers the 27
+// pre-collision populations of its site from the 27 neighbours x - c_i (periodic wrap;
+// consecutive threads read consecutive addresses of every plane, so each warp-wide load is one
+// coalesced row segment), collides in registers and writes the 27 post-collision values to
+// its own site of the other buffer (27 coalesced stores).
 // Algorithmic traffic per site update: 27 populations read + 27 written (216 bytes in
 // float32, 108 bytes in 16-bit storage).
+// On large boxes the TMA kernels are faster. On small ones, whose grid is resident at once, a step
+// lasts as long as its chain of launch, wait, loads, collision and stores, and plain loads and
+// stores make the shortest one. Microseconds per step of 16^3 / 32^3 / 48^3, float32 with noise: 6.2 /
+// 6.2 / 8.2 launched after the previous step had ended, 2.6 / 7.6 / 8.0 with dependent launch
+// and the draw behind the wait, 2.0 / 4.3 / 5.1 as it is; the row-segment TMA kernel takes 6.5 at
+// 32^3. Blocks of 64 threads spread a small box over the SMs (of 256: 2.4 / 4.4 / 5.2).
 #include "rflbm_internal.h"
+#include "tma.cuh"
 
 namespace rflbm_dev {
 
@@ -19,8 +26,15 @@ __global__ void __launch_bounds__(kStepBlock) step_pull(const StepParams p) {
   using T = typename S::T;
   // local site s of the launched rows (see StepParams); a z-slab's buffer holds it zlo rows up
   const uint32_t q = blockIdx.x * kStepBlock + threadIdx.x;
+  grid_launch_dependents();
   if (q >= p.nrows * p.geo.nx) return;
   const uint32_t s = p.row0 * p.geo.nx + q + (q >= p.row_split * p.geo.nx ? p.row_gap * p.geo.nx : 0u);
+  SiteNoise noise;
+  if (kNoise) {
+    site_noise_part<0, 6>(s + p.geo.site0, p.step, p.replica, p.rk, noise);
+    if (!normals_formed<24>(noise)) return;
+  }
+  grid_dependency_wait();
   const PullDeltas d = pull_deltas(s, p.geo);
   const int64_t sb = s + (int64_t)p.geo.zlo * p.geo.nxy;
   const T* __restrict__ src = static_cast<const T*>(p.src) + sb;
@@ -32,9 +46,6 @@ __global__ void __launch_bounds__(kStepBlock) step_pull(const StepParams p) {
     G[cx_of(i) + 1][cy_of(i) + 1][cz_of(i) + 1] =
         S::load(__ldg((src + pull_delta(d, i)) + plane_of(i) * p.geo.ps), class_of(i), p.ss);
   }
-
-  SiteNoise noise;
-  if (kNoise) site_noise(s + p.geo.site0, p.step, p.replica, p.key0, p.key1, noise);
 
   collide_site<kModel, kNoise, kGhostNeq, kPhiRho0>(G, p.cp, noise);
 
@@ -52,11 +63,18 @@ __global__ void __launch_bounds__(kStepBlock) step_aa_gather(const StepParams p)
   using S = Storage<kStore>;
   using T = typename S::T;
   const uint32_t q = blockIdx.x * kStepBlock + threadIdx.x;
+  grid_launch_dependents();
   if (q >= p.nrows * p.geo.nx) return;
   const uint32_t s = p.row0 * p.geo.nx + q + (q >= p.row_split * p.geo.nx ? p.row_gap * p.geo.nx : 0u);
   T* const buf = static_cast<T*>(p.dst) + s + (int64_t)p.geo.zlo * p.geo.nxy;
   PullDeltas d{};
   if (kOdd) d = pull_deltas(s, p.geo);
+  SiteNoise noise;
+  if (kNoise) {
+    site_noise_part<0, 6>(s + p.geo.site0, p.step, p.replica, p.rk, noise);
+    if (!normals_formed<24>(noise)) return;
+  }
+  grid_dependency_wait();
 
   float G[3][3][3];
 #pragma unroll
@@ -66,9 +84,6 @@ __global__ void __launch_bounds__(kStepBlock) step_aa_gather(const StepParams p)
                             : (int64_t)plane_of(i) * p.geo.ps;
     G[cx_of(i) + 1][cy_of(i) + 1][cz_of(i) + 1] = S::load(buf[at], class_of(i), p.ss);
   }
-
-  SiteNoise noise;
-  if (kNoise) site_noise(s + p.geo.site0, p.step, p.replica, p.key0, p.key1, noise);
 
   collide_site<kModel, kNoise, false, false>(G, p.cp, noise);
 
@@ -81,11 +96,22 @@ __global__ void __launch_bounds__(kStepBlock) step_aa_gather(const StepParams p)
   }
 }
 
+static cudaError_t launch_general(void (*kernel)(StepParams), const StepParams& p, cudaStream_t stream) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((p.nrows * p.geo.nx + kStepBlock - 1) / kStepBlock);
+  cfg.blockDim = dim3(kStepBlock);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, p);
+}
+
 template <int kStore, bool kOdd, int kModel, bool kNoise>
 static cudaError_t launch_aa(const StepParams& p, cudaStream_t stream) {
-  const uint32_t blocks = (p.nrows * p.geo.nx + kStepBlock - 1) / kStepBlock;
-  step_aa_gather<kStore, kOdd, kModel, kNoise><<<blocks, kStepBlock, 0, stream>>>(p);
-  return cudaGetLastError();
+  return launch_general(step_aa_gather<kStore, kOdd, kModel, kNoise>, p, stream);
 }
 
 template <int kStore, bool kOdd>
@@ -114,9 +140,7 @@ cudaError_t launch_step_aa_gather(const StepParams& p, const StepVariant& v, boo
 
 template <int kStore, int kModel, bool kNoise, bool kGhostNeq, bool kPhiRho0>
 static cudaError_t launch(const StepParams& p, cudaStream_t stream) {
-  const uint32_t blocks = (p.nrows * p.geo.nx + kStepBlock - 1) / kStepBlock;
-  step_pull<kStore, kModel, kNoise, kGhostNeq, kPhiRho0><<<blocks, kStepBlock, 0, stream>>>(p);
-  return cudaGetLastError();
+  return launch_general(step_pull<kStore, kModel, kNoise, kGhostNeq, kPhiRho0>, p, stream);
 }
 
 // 16-bit storage supports the paper's configuration (omega_g = 1, local rho in Eq. 10).
