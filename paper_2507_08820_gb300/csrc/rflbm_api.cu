@@ -284,10 +284,12 @@ bool setup_flat(rflbm* h) {
 // 128x32x32 (131,072 sites) 6.3 and 6.6. Without noise float32 32^3 6.2 and 5.1, 96x32x32 6.1 and
 // 6.0; 16-bit 32^3 5.6 and 6.0.
 // Rows that no segment width divides: 56^3 (ragged segments) 9.2 and 8.5, without noise 9.6 and 6.3;
-// 80^3 without noise 17.9 and 15.8.
+// 80^3 without noise 17.9 and 15.8. Ragged segments of 128 sites and more without noise in 16-bit
+// storage are like whole ones (128x32x32 5.2 and 7.0).
 bool general_pays(const rflbm* h) {
   if (h->slab || h->cfg.kernel != RFLBM_KERNEL_AUTO) return false;
   const bool noise = h->variant.noise, f32 = h->variant.storage == kStoreF32;
+  if (tma_segment_width(h->geo.nx) == 0 && !noise && !f32 && tma_ragged_width(h->geo.nx, 2) >= 128) return false;
   if (tma_segment_width(h->geo.nx) == 0) return h->geo.n < (noise ? 190000u : (f32 ? 450000u : 230000u));
   return noise ? h->geo.n < 112000u : (f32 && h->geo.n < 60000u);
 }

@@ -25,8 +25,8 @@ bool flat_pays(const Geometry& g, const StepVariant& v, bool aa) {
   const bool f32 = v.storage == kStoreF32;
   switch (tma_segment_width(g.nx)) {
     case 0: {
-      const int w = tma_ragged_width(g.nx, storage_bytes(v.storage));
-      const bool wide = w >= 128, full = wide && (g.nx + w - 1) / w * w * 30 <= g.nx * 31;
+      const uint64_t nx = g.nx, w = (uint64_t)tma_ragged_width(g.nx, storage_bytes(v.storage));
+      const bool wide = w >= 128, full = wide && (nx + w - 1) / w * w * 30 <= nx * 31;
       if (full || (wide && !f32 && !v.noise && !aa)) return false;
       if (!v.noise) return g.n >= (f32 ? 450000u : 230000u);
       return g.n >= (w && f32 && !aa ? 250000u : 200000u);
