@@ -97,9 +97,19 @@ __device__ __forceinline__ float lg2_approx(float x) {
 // e = 1 - u0 = (~x0 + 1/2) 2^-32 formed exactly from the integer, by the series
 // e + e^2/2 + e^3/3 when e < 2^-8 (truncation below 2e-8 relative) and by log2 otherwise,
 // so that radii near 0 keep their relative accuracy; log2 near 1 has an absolute error
-// near 2^-22, which for e >= 2^-8 is a radius error below 2e-6 absolute.
+// near 2^-22, which for e >= 2^-8 is a radius error below 2e-6 absolute. e < 2^-8 holds for
+// x0 > 0xFF000000 only (the e of that word rounds to 2^-8): one integer comparison (float16 256^3
+// 510 -> 504 us per step against the comparison of e).
 // The angle is taken in (-pi, pi] where __sincosf is accurate: 2 pi u1 - pi, whose
 // cosine and sine are the negatives of those of 2 pi u1.
+__device__ __forceinline__ void box_muller_direction(uint32_t x1, float& c, float& s) {
+  const float t = fmaf(__uint2float_rn(x1), 6.283185307179586f * 0x1p-32f,
+                       6.283185307179586f * 0x1p-33f - 3.14159265358979f);
+  float st, ct;
+  __sincosf(t, &st, &ct);
+  c = -ct;
+  s = -st;
+}
 __device__ __forceinline__ void box_muller(uint32_t x0, uint32_t x1, float& r, float& c,
                                            float& s) {
   const bool upper = (x0 >> 31) != 0u;
@@ -108,13 +118,8 @@ __device__ __forceinline__ void box_muller(uint32_t x0, uint32_t x1, float& r, f
   const float arg = upper ? 1.0f - e : e;
   const float lg = -1.3862943611198906f * lg2_approx(arg);  // -2 ln(arg)
   const float ser = e * fmaf(e, fmaf(e, 0.66666667f, 1.0f), 2.0f);  // 2e + e^2 + 2e^3/3
-  r = sqrt_approx((upper && e < 0.00390625f) ? ser : lg);
-  const float t = fmaf(__uint2float_rn(x1), 6.283185307179586f * 0x1p-32f,
-                       6.283185307179586f * 0x1p-33f - 3.14159265358979f);
-  float st, ct;
-  __sincosf(t, &st, &ct);
-  c = -ct;
-  s = -st;
+  r = sqrt_approx(x0 > 0xFF000000u ? ser : lg);  // (upper and e < 2^-8)
+  box_muller_direction(x1, c, s);
 }
 
 // The 24 normals of one site at one step: Box-Muller pair m of call j (m = 2j, 2j + 1)
@@ -123,10 +128,42 @@ struct SiteNoise {
   float n[24];
 };
 
+// The radius of box_muller, the same bits, with its two-way choices as predicated instructions
+// instead of selections: on GB300 an ALU instruction (select, compare, logic, conversion) takes
+// twice the issue slots of a float32 one, and a step's 12 pairs leave 48 of them. Used by the
+// one-site kernels (float32 128^3 70.0 -> 68.8 us per step, 256^3 535.7 -> 526.3; the draw alone 44.4 ->
+// 46.5 G sites/s); the two-site kernels measured slower with it (float16 256^3 510 -> 522 us).
+__device__ __forceinline__ float box_muller_radius(uint32_t x0) {
+  float r;
+  asm("{\n\t"
+      ".reg .pred p, q;\n\t"
+      ".reg .b32 xm;\n\t"
+      ".reg .f32 e, s, lg;\n\t"
+      "setp.lt.s32 p, %1, 0;\n\t"
+      "setp.gt.u32 q, %1, 0xFF000000;\n\t"
+      "mov.b32 xm, %1;\n\t"
+      "@p not.b32 xm, xm;\n\t"
+      "cvt.rn.f32.u32 e, xm;\n\t"
+      "fma.rn.f32 e, e, 0f2F800000, 0f2F000000;\n\t"   // 2^-32, 2^-33
+      "fma.rn.f32 s, e, 0f3F2AAAAB, 0f3F800000;\n\t"   // the series 2e + e^2 + 2e^3/3
+      "fma.rn.f32 s, e, s, 0f40000000;\n\t"
+      "mul.rn.f32 s, e, s;\n\t"
+      "@p sub.rn.f32 e, 0f3F800000, e;\n\t"
+      "lg2.approx.ftz.f32 lg, e;\n\t"
+      "mul.rn.f32 lg, lg, 0fBFB17218;\n\t"             // -2 ln 2
+      "@q mov.b32 lg, s;\n\t"
+      "sqrt.approx.ftz.f32 %0, lg;\n\t"
+      "}"
+      : "=f"(r)
+      : "r"(x0));
+  return r;
+}
+
 // The two normals of one Box-Muller pair.
 __device__ __forceinline__ void box_muller_normals(uint32_t x0, uint32_t x1, float& n0, float& n1) {
-  float r, c, s;
-  box_muller(x0, x1, r, c, s);
+  const float r = box_muller_radius(x0);
+  float c, s;
+  box_muller_direction(x1, c, s);
   n0 = __fmul_rn(r, c);
   n1 = __fmul_rn(r, s);
 }
