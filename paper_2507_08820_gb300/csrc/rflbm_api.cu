@@ -26,6 +26,7 @@ struct HostResults {
   int err;
   double stats[kStatOutFields];
   double modes[2 * kQ];
+  unsigned spectrum_range;
 };
 
 struct rflbm {
@@ -66,7 +67,8 @@ struct rflbm {
   int host_shells_n = 0;          // shells it holds
   void* diag_spec = nullptr;      // its half spectrum
   SpectrumAxis axes[3];           // the library's transform
-  float4* twiddles = nullptr;     // their tables
+  float4* twiddles = nullptr;     // their tables, and the range word of a transform
+  unsigned* spectrum_range = nullptr;
   cufftHandle fft_plan = 0;       // cuFFT's, where an edge is none of the library's lengths
   bool own_fft = false;
   bool fft_ready = false;
@@ -548,7 +550,7 @@ void rflbm_destroy(rflbm_t* h) {
   cudaFree(h->diag_partials);
   cudaFree(h->diag_field);
   cudaFree(h->diag_spec);
-  if (h->fft_ready && !h->own_fft) cufftDestroy(h->fft_plan);
+  if (h->fft_ready) cufftDestroy(h->fft_plan);
   cudaFree(h->twiddles);
   cudaFree(h->staging);
   if (h->faces_ready) cudaEventDestroy(h->faces_ready);
@@ -869,32 +871,30 @@ int rflbm_structure_factor(rflbm_t* h, int field, int nshell, double* s_sum, dou
   DeviceGuard guard(h->device);
   const Geometry& g = h->geo;
   const size_t nspec = (size_t)g.nz * g.ny * (g.nx / 2 + 1);
-  if (!h->fft_ready) {
-    if (!h->diag_field)
-      RFLBM_CUDA(cudaMalloc((void**)&h->diag_field, sizeof(double) * g.n), "allocating the field buffer");
-    if (!h->diag_spec)
-      RFLBM_CUDA(cudaMalloc(&h->diag_spec, sizeof(cufftDoubleComplex) * nspec), "allocating the spectrum");
-    const int edge[3] = {(int)g.nx, (int)g.ny, (int)g.nz};
-    h->own_fft = true;
-    for (int a = 0; a < 3; ++a) h->own_fft = spectrum_axis(edge[a], &h->axes[a]) && h->own_fft;
-    if (h->own_fft) {
+  if (!h->diag_field)
+    RFLBM_CUDA(cudaMalloc((void**)&h->diag_field, sizeof(double) * g.n), "allocating the field buffer");
+  if (!h->diag_spec)
+    RFLBM_CUDA(cudaMalloc(&h->diag_spec, sizeof(cufftDoubleComplex) * nspec), "allocating the spectrum");
+  const int edge[3] = {(int)g.nx, (int)g.ny, (int)g.nz};
+  if (!h->own_fft && !h->fft_ready) {
+    bool own = true;
+    for (int a = 0; a < 3; ++a) own = spectrum_axis(edge[a], &h->axes[a]) && own;
+    if (own) {
       std::vector<float> table;
       for (int a = 0; a < 3; ++a) {
         const std::vector<float> t = spectrum_twiddles(edge[a]);
         table.insert(table.end(), t.begin(), t.end());
       }
-      if (!h->twiddles)
-        RFLBM_CUDA(cudaMalloc((void**)&h->twiddles, sizeof(float) * table.size()), "allocating the twiddle factors");
-      RFLBM_CUDA(cudaMemcpy(h->twiddles, table.data(), sizeof(float) * table.size(), cudaMemcpyHostToDevice),
-                 "copying the twiddle factors");
-      for (int a = 0, at = 0; a < 3; at += edge[a++]) h->axes[a].twiddles = h->twiddles + at;
-    } else if (cufftPlan3d(&h->fft_plan, edge[2], edge[1], edge[0], CUFFT_D2Z) != CUFFT_SUCCESS) {
-      return fail(RFLBM_ECUDA, "cufftPlan3d failed for %u x %u x %u", g.nx, g.ny, g.nz);
+      table.resize(table.size() + 4, 0.0f);  // the range word, zero
+      const size_t bytes = sizeof(float) * table.size();
+      if (!h->twiddles) RFLBM_CUDA(cudaMalloc((void**)&h->twiddles, bytes), "allocating the twiddle factors");
+      RFLBM_CUDA(cudaMemcpy(h->twiddles, table.data(), bytes, cudaMemcpyHostToDevice), "copying the twiddle factors");
+      int at = 0;
+      for (int a = 0; a < 3; at += edge[a++]) h->axes[a].twiddles = h->twiddles + at;
+      h->spectrum_range = reinterpret_cast<unsigned*>(h->twiddles + at);
+      h->own_fft = true;
     }
-    h->fft_ready = true;
   }
-  if (!h->own_fft && cufftSetStream(h->fft_plan, h->stream) != CUFFT_SUCCESS)
-    return fail(RFLBM_ECUDA, "cufftSetStream failed");
   const int blocks = std::max(1, std::min(4 * std::max(h->num_sms, 1), (int)((nspec + 255) / 256)));
   if (int e = ensure_diag_partials(h, sizeof(double) * (size_t)blocks * 2 * nshell)) return e;
   if (h->host_shells_n < nshell) {
@@ -907,23 +907,35 @@ int rflbm_structure_factor(rflbm_t* h, int field, int nshell, double* s_sum, dou
   }
   const double* const host = h->host_shells;
   const void* const src = h->buf[h->cur];
+  bool done = false;
   if (h->own_fft) {
     float* const field_values = reinterpret_cast<float*>(h->diag_field);
+    float2* const power = reinterpret_cast<float2*>(h->diag_field);
     RFLBM_CUDA(launch_field(vgeo(h), h->ss, h->variant.storage, src, field, field_values, h->stream),
                "launching the field kernel");
-    RFLBM_CUDA(launch_power_spectrum(g, h->axes, field_values, h->diag_spec, h->diag_field, h->stream),
+    RFLBM_CUDA(launch_power_spectrum(g, h->axes, field_values, h->diag_spec, power, h->spectrum_range, h->stream),
                "launching the spectrum kernels");
-    RFLBM_CUDA(launch_power_bins(g, h->diag_field, nshell, blocks, h->diag_partials, h->host_shells, h->stream),
+    RFLBM_CUDA(launch_power_bins(g, power, nshell, blocks, h->diag_partials, h->host_shells, h->spectrum_range,
+                                 &h->host->spectrum_range, h->stream),
                "launching the shell binning");
-  } else {
+    if (int e = sync(h, "rflbm_structure_factor")) return e;
+    done = spectrum_usable(h->host->spectrum_range);
+  }
+  if (!done) {  // edges that are none of the library's lengths, fields whose squares leave float32
+    if (!h->fft_ready) {
+      if (cufftPlan3d(&h->fft_plan, edge[2], edge[1], edge[0], CUFFT_D2Z) != CUFFT_SUCCESS)
+        return fail(RFLBM_ECUDA, "cufftPlan3d failed for %u x %u x %u", g.nx, g.ny, g.nz);
+      h->fft_ready = true;
+    }
+    if (cufftSetStream(h->fft_plan, h->stream) != CUFFT_SUCCESS) return fail(RFLBM_ECUDA, "cufftSetStream failed");
     RFLBM_CUDA(launch_field(vgeo(h), h->ss, h->variant.storage, src, field, h->diag_field, h->stream),
                "launching the field kernel");
     if (cufftExecD2Z(h->fft_plan, h->diag_field, (cufftDoubleComplex*)h->diag_spec) != CUFFT_SUCCESS)
       return fail(RFLBM_ECUDA, "cufftExecD2Z failed");
     RFLBM_CUDA(launch_shell_bins(g, h->diag_spec, nshell, blocks, h->diag_partials, h->host_shells, h->stream),
                "launching the shell binning");
+    if (int e = sync(h, "rflbm_structure_factor")) return e;
   }
-  if (int e = sync(h, "rflbm_structure_factor")) return e;
   for (int n = 0; n < nshell; ++n) {
     s_sum[n] = host[n];
     count[n] = host[nshell + n];

@@ -120,9 +120,14 @@ __global__ void __launch_bounds__(kDiagBlock, 2) k_mode_sums(Geometry g, StoreSc
 // Column sums of a row-major array in a fixed order: a block per column, thread t adds rows
 // t, t + 256, ..., then a fixed tree.
 __global__ void __launch_bounds__(kDiagBlock) k_reduce_columns(const double* __restrict__ partials, int64_t rows, int cols,
-                                 double* __restrict__ out) {
+                                 double* __restrict__ out, unsigned* range = nullptr,
+                                 unsigned* range_out = nullptr) {
   __shared__ double sh[kDiagBlock / 32];
   const int col = blockIdx.x;
+  if (range && col == 0 && threadIdx.x == 0) {
+    *range_out = *range;
+    *range = 0u;
+  }
   double v = 0.0;
   for (int64_t r = threadIdx.x; r < rows; r += kDiagBlock) v += partials[r * cols + col];
 #pragma unroll
@@ -177,20 +182,31 @@ __device__ __forceinline__ int shell_of(int kx, int ky, int kz, const Geometry& 
   return (int)llrint(L * sqrt(fx * fx + fy * fy + fz * fz));
 }
 
-// |F|^2 of one entry of a spectrum: of its complex value, or given.
+// |F|^2 of one entry of a spectrum and the sums of a scan: float32 pairs where they are given, FP64
+// for cuFFT's complex values.
 __device__ __forceinline__ double power_of(const cufftDoubleComplex& c) { return fma(c.x, c.x, c.y * c.y); }
-__device__ __forceinline__ double power_of(double p) { return p; }
+__device__ __forceinline__ Pair32 power_of(float2 p) { return {p.x, p.y}; }
+__device__ __forceinline__ double twice(double v) { return 2.0 * v; }
+__device__ __forceinline__ Pair32 twice(Pair32 v) { return {2.0f * v.hi, 2.0f * v.lo}; }
+__device__ __forceinline__ double scan_add(double a, double b) { return a + b; }
+__device__ __forceinline__ Pair32 scan_add(Pair32 a, Pair32 b) { return padd(a, b); }
+__device__ __forceinline__ double from_lane(double v, int o) { return __shfl_up_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ Pair32 from_lane(Pair32 v, int o) {
+  return {__shfl_up_sync(0xffffffffu, v.hi, o), __shfl_up_sync(0xffffffffu, v.lo, o)};
+}
+__device__ __forceinline__ double fp64_of(double v) { return v; }
+__device__ __forceinline__ double fp64_of(Pair32 v) { return (double)v.hi + (double)v.lo; }
 
 // Shell sums of |F(k)|^2 / N over the half spectrum of a real transform (kx = 0 .. nx/2),
 // each non-redundant vector counted twice. Shell n = round(|k| L / 2 pi) with
 // L = max(nx, ny, nz). The sums are reproducible bit for bit: each warp owns a row of
 // shell bins in shared memory. Along a spectrum row (ky, kz) the shell grows with kx, so the
 // vectors of one shell are neighbours: a segmented scan over the warp's lanes adds them up
-// (a fixed tree), and the last lane of each run adds the run to its bin, one spectrum row after
-// another. The rows are then summed in warp order into the block's partial row. (Counts are
-// integers, exact in any order.) Nine FP64 operations per vector; with the shell computed in
-// FP64 (three quotients and a root) and the lanes adding to the bins one after another, 128^3
-// took 190 us.
+// (a fixed tree of float32 pairs), and the last lane of each run adds the run to its FP64 bin, one
+// spectrum row after another. The rows are then summed in warp order into the block's partial
+// row. (Counts are integers, exact in any order.) Four FP64 operations per warp of vectors; with the
+// shell computed in FP64 (three quotients and a root) and the lanes adding to the bins one after
+// another 128^3 took 190 us, with the scan in FP64 28 us, so 17 us.
 template <class Entry>
 __global__ void __launch_bounds__(kDiagBlock) k_shell_bins(Geometry g, FastDiv div_nxh, FastDiv div_ny,
                                                            const Entry* __restrict__ spec, int nshell,
@@ -206,14 +222,13 @@ __global__ void __launch_bounds__(kDiagBlock) k_shell_bins(Geometry g, FastDiv d
   const int nxh = g.nx / 2 + 1;
   const int64_t total = (int64_t)g.nz * g.ny * nxh;  // at most n
   const double L = (double)max(g.nx, max(g.ny, g.nz));
-  const double inv_n = 1.0 / (double)g.n;
   const unsigned upto = 0xffffffffu >> (31 - lane);  // lanes 0 .. lane
   const int64_t stride = (int64_t)gridDim.x * kDiagBlock;
   for (int64_t wbase = (int64_t)blockIdx.x * kDiagBlock + 32 * wid; wbase < total; wbase += stride) {
     const int64_t idx = wbase + lane;  // warp-uniform trip count
     int shell = nshell;
     uint32_t row = 0xffffffffu;
-    double v = 0.0;
+    decltype(power_of(Entry())) v{};
     bool self = false;
     if (idx < total) {
       row = fastdiv((uint32_t)idx, div_nxh);
@@ -223,7 +238,8 @@ __global__ void __launch_bounds__(kDiagBlock) k_shell_bins(Geometry g, FastDiv d
       shell = min(nshell, shell_of(kx, ky <= (int)g.ny / 2 ? ky : ky - (int)g.ny,
                                    kz <= (int)g.nz / 2 ? kz : kz - (int)g.nz, g, L));
       self = (kx == 0) || ((g.nx % 2 == 0) && kx == (int)g.nx / 2);
-      v = power_of(spec[idx]) * (self ? inv_n : 2.0 * inv_n);
+      v = power_of(spec[idx]);
+      if (!self) v = twice(v);
     }
     const int before = __shfl_up_sync(0xffffffffu, shell, 1);
     const uint32_t row_before = __shfl_up_sync(0xffffffffu, row, 1);
@@ -232,8 +248,8 @@ __global__ void __launch_bounds__(kDiagBlock) k_shell_bins(Geometry g, FastDiv d
     const int start = 31 - __clz(heads & upto);  // first lane of this lane's run
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      const double t = __shfl_up_sync(0xffffffffu, v, o);
-      if (lane - o >= start) v += t;
+      const auto t = from_lane(v, o);
+      if (lane - o >= start) v = scan_add(v, t);
     }
     const bool tail = (lane == 31 || ((heads >> (lane + 1)) & 1u)) && shell < nshell;
     if (tail) {
@@ -244,14 +260,16 @@ __global__ void __launch_bounds__(kDiagBlock) k_shell_bins(Geometry g, FastDiv d
     const uint32_t first = __shfl_sync(0xffffffffu, row, 0);
     const uint32_t end = min(fastdiv((uint32_t)min(wbase + 31, total - 1), div_nxh), first + 31u);
     for (uint32_t r = first; r <= end; ++r) {
-      if (tail && row == r) mine[shell] += v;
+      if (tail && row == r) mine[shell] += fp64_of(v);
       __syncwarp();
     }
   }
   __syncthreads();
+  const double inv_n = 1.0 / (double)g.n;
   for (int j = threadIdx.x; j < nshell; j += kDiagBlock) {
     double sum = 0.0;
     for (int k = 0; k < kWarps; ++k) sum += bins[(size_t)k * nshell + j];
+    sum *= inv_n;
     partials[(int64_t)blockIdx.x * 2 * nshell + j] = sum;
     partials[(int64_t)blockIdx.x * 2 * nshell + nshell + j] = (double)counts[j];
   }
@@ -274,7 +292,7 @@ cudaError_t launch_mode_sums(const Geometry& g, const StoreScale& ss, int kind, 
     case kStoreBF16: k_mode_sums<kStoreBF16><<<(unsigned)blocks, kDiagBlock, 0, st>>>(g, ss, (const DT<kStoreBF16>*)src, partials); break;
     default: return cudaErrorInvalidValue;
   }
-  k_reduce_columns<<<2 * kQ, kDiagBlock, 0, st>>>(partials, blocks, 2 * kQ, out54);
+  k_reduce_columns<<<2 * kQ, kDiagBlock, 0, st>>>(partials, blocks, 2 * kQ, out54, nullptr, nullptr);
   return cudaGetLastError();
 }
 
@@ -312,7 +330,7 @@ cudaError_t launch_field(const Geometry& g, const StoreScale& ss, int kind, cons
 
 template <class Entry>
 static cudaError_t launch_bins(const Geometry& g, const Entry* spec, int nshell, int blocks, double* partials, double* out,
-                               cudaStream_t st) {
+                               unsigned* range, unsigned* range_out, cudaStream_t st) {
   // kDiagBlock / 32 rows of sums + one row of counts: up to 221 KB at nshell = 3072
   const size_t smem = sizeof(double) * (size_t)(kDiagBlock / 32 + 1) * (size_t)nshell;
   if (smem > 48 * 1024) {
@@ -321,16 +339,16 @@ static cudaError_t launch_bins(const Geometry& g, const Entry* spec, int nshell,
     if (e != cudaSuccess) return e;
   }
   k_shell_bins<<<blocks, kDiagBlock, smem, st>>>(g, make_fastdiv(g.nx / 2 + 1), make_fastdiv(g.ny), spec, nshell, partials);
-  k_reduce_columns<<<2 * nshell, kDiagBlock, 0, st>>>(partials, blocks, 2 * nshell, out);
+  k_reduce_columns<<<2 * nshell, kDiagBlock, 0, st>>>(partials, blocks, 2 * nshell, out, range, range_out);
   return cudaGetLastError();
 }
 cudaError_t launch_shell_bins(const Geometry& g, const void* spec, int nshell, int blocks,
                               double* partials, double* out, cudaStream_t st) {
-  return launch_bins(g, (const cufftDoubleComplex*)spec, nshell, blocks, partials, out, st);
+  return launch_bins(g, (const cufftDoubleComplex*)spec, nshell, blocks, partials, out, nullptr, nullptr, st);
 }
-cudaError_t launch_power_bins(const Geometry& g, const double* power, int nshell, int blocks, double* partials,
-                              double* out, cudaStream_t st) {
-  return launch_bins(g, power, nshell, blocks, partials, out, st);
+cudaError_t launch_power_bins(const Geometry& g, const float2* power, int nshell, int blocks, double* partials,
+                              double* out, unsigned* range, unsigned* range_out, cudaStream_t st) {
+  return launch_bins(g, power, nshell, blocks, partials, out, range, range_out, st);
 }
 
 }  // namespace rflbm_dev

@@ -19,10 +19,12 @@ cudaError_t launch_field(const Geometry& g, const StoreScale& ss, int kind, cons
 cudaError_t launch_field(const Geometry& g, const StoreScale& ss, int kind, const void* src,
                          int field, double* out, cudaStream_t st);
 // Shell sums of |F|^2 / N and vector counts of a half spectrum: out[n], out[nshell + n]. From a
-// D2Z spectrum, or from |F|^2.
+// D2Z spectrum, or from |F|^2 as float32 pairs (hi, lo); then *range goes to *range_out and is
+// zeroed.
 cudaError_t launch_shell_bins(const Geometry& g, const void* spec, int nshell, int blocks,
                               double* partials, double* out, cudaStream_t st);
-cudaError_t launch_power_bins(const Geometry& g, const double* power, int nshell, int blocks,
-                              double* partials, double* out, cudaStream_t st);
+cudaError_t launch_power_bins(const Geometry& g, const float2* power, int nshell, int blocks,
+                              double* partials, double* out, unsigned* range, unsigned* range_out,
+                              cudaStream_t st);
 
 }  // namespace rflbm_dev

@@ -12,7 +12,7 @@
 // radix 8, 4, 2 and the odd primes up to 13, two buffers):
 //   x: two real rows at a time as one complex line; the half spectra of both rows out
 //   y: in place
-//   z: the last transform, and |F|^2 in FP64 out instead of the spectrum
+//   z: the last transform, and |F|^2 out instead of the spectrum
 // The spectrum between the passes is read and written once each and stays in L2 up to 192^3.
 #include "rflbm_spectrum.h"
 #include "wide.cuh"
@@ -204,10 +204,11 @@ __global__ void __launch_bounds__(256) k_spectrum_x(const __grid_constant__ Spec
 }
 
 // Lines of n values `inner` apart: line l = (l / inner, l % inner) starts at (l / inner) n inner +
-// l % inner. In place, or |F|^2 in FP64 to `power`.
+// l % inner. In place, or |F|^2 (hi, lo) to `power`.
 template <int kOdd, bool kPower>
 __global__ void __launch_bounds__(256) k_spectrum_lines(const __grid_constant__ SpectrumAxis ax, float4* __restrict__ spec, uint32_t lines,
-                                                         FastDiv inner, double* __restrict__ power) {
+                                                         FastDiv inner, float2* __restrict__ power,
+                                                         unsigned* __restrict__ range) {
   extern __shared__ float4 smem[];
   const int n = ax.n;
   float4 *a = smem, *b = smem + n * kCols, *tw = smem + 2 * n * kCols;
@@ -221,16 +222,24 @@ __global__ void __launch_bounds__(256) k_spectrum_lines(const __grid_constant__ 
     a[i * kCols + c] = l < lines ? spec[at + (int64_t)i * inner.d] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   __syncthreads();
   a = transform<kOdd>(a, b, tw, ax);
-  if (l >= lines) return;
-  for (int i = threadIdx.x / kCols; i < n; i += blockDim.x / kCols) {
+  unsigned seen = 0u;
+  for (int i = threadIdx.x / kCols; i < n && l < lines; i += blockDim.x / kCols) {
     const float4 v = a[i * kCols + c];
     if (kPower) {
       const Cpx f = unpack(v);
       const Pair32 q = padd(pmul(f.re, f.re), pmul(f.im, f.im));
-      power[at + (int64_t)i * inner.d] = (double)q.hi + (double)q.lo;
+      power[at + (int64_t)i * inner.d] = make_float2(q.hi, q.lo);
+      const float most = fmaxf(fabsf(v.x), fabsf(v.z));
+      // (a NaN is lost by fmaxf: its sum is not)
+      seen |= (v.x + v.z < 0x1p60f && v.x + v.z > -0x1p60f && most < 0x1p60f ? 0u : kSpectrumLarge) |
+              (most >= 0x1p-30f ? kSpectrumUsual : 0u) | (most > 0.0f ? kSpectrumNonzero : 0u);
     } else {
       spec[at + (int64_t)i * inner.d] = v;
     }
+  }
+  if (kPower) {
+    seen = __reduce_or_sync(0xffffffffu, seen);
+    if ((threadIdx.x & 31) == 0 && (seen & ~*(volatile unsigned*)range)) atomicOr(range, seen);
   }
 }
 
@@ -280,14 +289,14 @@ std::vector<float> spectrum_twiddles(int n) {
 }
 
 cudaError_t launch_power_spectrum(const Geometry& g, const SpectrumAxis (&ax)[3], const float* field, void* spec,
-                                  double* power, cudaStream_t st) {
+                                  float2* power, unsigned* range, cudaStream_t st) {
   const int64_t rows = (int64_t)g.ny * g.nz;
   const uint32_t nh = g.nx / 2 + 1;
   float4* const s = static_cast<float4*>(spec);
   const auto lines = [&](auto* kernel, const SpectrumAxis& a, uint32_t nlines, uint32_t inner) {
     const size_t smem = line_smem(a.n);
     if (cudaError_t e = allow_smem(kernel, smem)) return e;
-    kernel<<<(nlines + kCols - 1) / kCols, line_threads(a.n), smem, st>>>(a, s, nlines, make_fastdiv(inner), power);
+    kernel<<<(nlines + kCols - 1) / kCols, line_threads(a.n), smem, st>>>(a, s, nlines, make_fastdiv(inner), power, range);
     return cudaGetLastError();
   };
   const auto first = [&](auto* kernel) {

@@ -20,9 +20,17 @@ struct SpectrumAxis {
 bool spectrum_axis(int n, SpectrumAxis* ax);
 std::vector<float> spectrum_twiddles(int n);
 
-// |F|^2 of the half spectrum, [kz][ky][kx], kx <= nx / 2, from the field (one float per site). spec
+// What *range tells after a transform, as bits: some |F| is 2^60 or more or not finite; some |F| is
+// 2^-30 or more; some |F| is not zero. With kSpectrumLarge, or with kSpectrumNonzero alone, the
+// squares leave the range of float32 and the spectrum has to be taken in FP64 (spectrum_usable).
+enum : unsigned { kSpectrumLarge = 1u, kSpectrumUsual = 2u, kSpectrumNonzero = 4u };
+inline bool spectrum_usable(unsigned range) {
+  return !(range & kSpectrumLarge) && ((range & kSpectrumUsual) || !(range & kSpectrumNonzero));
+}
+
+// |F|^2 (hi, lo) of the half spectrum, [kz][ky][kx], kx <= nx / 2, from the field (one float per site). spec
 // holds 16 bytes per value; power may be the field's memory.
 cudaError_t launch_power_spectrum(const Geometry& g, const SpectrumAxis (&ax)[3], const float* field, void* spec,
-                                  double* power, cudaStream_t st);
+                                  float2* power, unsigned* range, cudaStream_t st);
 
 }  // namespace rflbm_dev

@@ -143,3 +143,30 @@ def test_shell_sums_of_uneven_boxes(R, shape, nshell):
         assert np.array_equal(got_c, want_c[:got_c.size]), k
         assert np.allclose(got_s, want_s[:got_s.size], rtol=1e-5, atol=1e-6 * want_s.max()), k
     box.close()
+
+
+@pytest.mark.parametrize("scale", [1e-25, 1e-12, 1e-3, 1e15, 1e25])
+@pytest.mark.parametrize("shape", [(24, 10, 9), (31, 4, 3)])
+def test_structure_factors_at_every_scale(R, scale, shape):
+    """Fields whose squares leave the range of float32 (and edges that are none of the library's
+    lengths) take cuFFT, usual ones the library's transform."""
+    f = _state(shape, 13, scale)
+    box = R.Box(*shape, tau=0.8, rho0=1e-30)
+    R.rflbm_set_populations(box.h, np.ascontiguousarray(f))
+    f = box.populations()
+    cx = o.velocities()[:, 0].astype(float)
+    ns = R.rflbm_shell_count(box.h)
+    got_s, _ = R.rflbm_structure_factor(box.h, 1)
+    again, _ = R.rflbm_structure_factor(box.h, 1)
+    box.close()
+    want_s, _ = _shells_numpy(cx @ f, shape, ns)
+    assert np.array_equal(got_s, again)
+    assert np.allclose(got_s, want_s, rtol=1e-4, atol=1e-5 * want_s.max())
+
+
+def test_structure_factor_of_a_fluid_at_rest_is_zero(R):
+    box = R.Box(24, 10, 9, tau=0.8)
+    R.rflbm_init_rest(box.h)
+    s, count = R.rflbm_structure_factor(box.h, 0)
+    box.close()
+    assert not s.any() and count.sum() == 24 * 10 * 9
