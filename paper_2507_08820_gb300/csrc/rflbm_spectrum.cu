@@ -13,7 +13,9 @@
 //   x: two real rows at a time as one complex line; the half spectra of both rows out
 //   y: in place
 //   z: the last transform, and |F|^2 out instead of the spectrum
-// The spectrum between the passes is read and written once each and stays in L2 up to 192^3.
+// The spectrum between the passes is read and written once each and stays in L2 up to 192^3. The
+// three passes of 128^3 took 24 + 21 + 23 us with the tile loaded to and stored from shared memory,
+// and 16 + 16 + 17 us with the first stage loading and the last one storing in global memory.
 #include "rflbm_spectrum.h"
 #include "wide.cuh"
 
@@ -117,9 +119,10 @@ __device__ __forceinline__ void dft(Cpx (&v)[R], const float4* tw, int step) {
 }
 
 // One Stockham stage of radix R over a tile of kCols lines: `before` is the product of the radices
-// done so far.
-template <int R>
-__device__ __forceinline__ void stage(const float4* in, float4* out, const float4* tw, int n, int before) {
+// done so far; load(position, line) and store(position, line, value) reach the tile. Consecutive
+// threads take consecutive lines.
+template <int R, class Load, class Store>
+__device__ __forceinline__ void stage(const Load& load, const Store& store, const float4* tw, int n, int before) {
   const int m = n / R;
   for (int b = threadIdx.x; b < m * kCols; b += blockDim.x) {
     const int c = b % kCols, j = b / kCols;
@@ -127,47 +130,64 @@ __device__ __forceinline__ void stage(const float4* in, float4* out, const float
     Cpx v[R];
     const int tstep = k * (m / before);  // twiddle exp(-2 pi i r k / (before R))
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      v[r] = unpack(in[(j + r * m) * kCols + c]);
-      if (r > 0 && before > 1) v[r] = cmul(v[r], unpack(tw[r * tstep]));
+    for (int r = 0; r < R; ++r) v[r] = load(j + r * m, c);
+    if (before > 1) {
+#pragma unroll
+      for (int r = 1; r < R; ++r) v[r] = cmul(v[r], unpack(tw[r * tstep]));
     }
     dft<R>(v, tw, m);
     const int o = q * before * R + k;
 #pragma unroll
-    for (int r = 0; r < R; ++r) out[(o + r * before) * kCols + c] = pack(v[r]);
+    for (int r = 0; r < R; ++r) store(o + r * before, c, v[r]);
   }
 }
 
-// The lines of a tile through all stages (a and b: n x kCols each); returns the buffer that holds
-// the result. Starts and ends with the tile visible to all threads. kOdd: 1 with the radices 3, 5
-// and 7, 2 with 11 and 13 too (64, 100 and 180 registers).
-template <int kOdd>
-__device__ __forceinline__ float4* transform(float4* a, float4* b, const float4* tw, const SpectrumAxis& ax) {
-  int before = 1;
-  for (int f = 0; f < ax.nfactors; ++f) {
-    const int r = ax.factors[f];
-    switch (r) {
-      case 8: stage<8>(a, b, tw, ax.n, before); break;
-      case 4: stage<4>(a, b, tw, ax.n, before); break;
-      case 2: stage<2>(a, b, tw, ax.n, before); break;
-      default:
-        if constexpr (kOdd > 0) {
-          if (r == 3) stage<3>(a, b, tw, ax.n, before);
-          if (r == 5) stage<5>(a, b, tw, ax.n, before);
-          if (r == 7) stage<7>(a, b, tw, ax.n, before);
-        }
-        if constexpr (kOdd > 1) {
-          if (r == 11) stage<11>(a, b, tw, ax.n, before);
-          if (r == 13) stage<13>(a, b, tw, ax.n, before);
-        }
-    }
-    before *= r;
+template <int kOdd, class Load, class Store>
+__device__ __forceinline__ void stage_of(int r, const Load& load, const Store& store, const float4* tw, int n, int before) {
+  if (r == 8) stage<8>(load, store, tw, n, before);
+  else if (r == 4) stage<4>(load, store, tw, n, before);
+  else if (r == 2) stage<2>(load, store, tw, n, before);
+  if constexpr (kOdd > 0) {
+    if (r == 3) stage<3>(load, store, tw, n, before);
+    if (r == 5) stage<5>(load, store, tw, n, before);
+    if (r == 7) stage<7>(load, store, tw, n, before);
+  }
+  if constexpr (kOdd > 1) {
+    if (r == 11) stage<11>(load, store, tw, n, before);
+    if (r == 13) stage<13>(load, store, tw, n, before);
+  }
+}
+
+// The lines of a tile through all stages: the first one loads from global memory, the last one
+// stores there (they keep no copy of the tile in shared memory, and their accesses overlap with
+// the butterflies); between stages the values go through the buffers a and b in turn. kOdd: 1 with
+// the radices 3, 5 and 7, 2 with 11 and 13 too.
+template <int kOdd, class Load, class Store>
+__device__ __forceinline__ void transform(float4* a, float4* b, const float4* tw, const SpectrumAxis& ax, const Load& load,
+                                          const Store& store) {
+  const int n = ax.n, last = ax.nfactors - 1;
+  if (last < 0) {  // n = 1
+    if (threadIdx.x < kCols) store(0, (int)threadIdx.x, load(0, (int)threadIdx.x));
+    return;
+  }
+  if (kOdd > 0) __syncthreads();  // odd radices read the twiddles in their first stage
+  if (last == 0) {
+    stage_of<kOdd>(ax.factors[0], load, store, tw, n, 1);
+    return;
+  }
+  stage_of<kOdd>(ax.factors[0], load, [&](int i, int c, const Cpx& v) { a[i * kCols + c] = pack(v); }, tw, n, 1);
+  __syncthreads();
+  int before = ax.factors[0];
+  for (int f = 1; f < last; ++f) {
+    stage_of<kOdd>(ax.factors[f], [&](int i, int c) { return unpack(a[i * kCols + c]); },
+                   [&](int i, int c, const Cpx& v) { b[i * kCols + c] = pack(v); }, tw, n, before);
+    before *= ax.factors[f];
     float4* const t = a;
     a = b;
     b = t;
     __syncthreads();
   }
-  return a;
+  stage_of<kOdd>(ax.factors[last], [&](int i, int c) { return unpack(a[i * kCols + c]); }, store, tw, n, before);
 }
 
 __device__ __forceinline__ void load_twiddles(float4* tw, const SpectrumAxis& ax) {
@@ -177,26 +197,29 @@ __device__ __forceinline__ void load_twiddles(float4* tw, const SpectrumAxis& ax
 // Rows 2 p and 2 p + 1 of the field (of `rows` rows of n values) as the real and imaginary parts of
 // line p; their half spectra to spec[row][kx], kx <= n / 2.
 template <int kOdd>
-__global__ void __launch_bounds__(256) k_spectrum_x(const __grid_constant__ SpectrumAxis ax, const float* __restrict__ field, int64_t rows,
+__global__ void __launch_bounds__(256) k_spectrum_x(const __grid_constant__ SpectrumAxis ax,
+                                                     const float* __restrict__ field, int64_t rows,
                                                      float4* __restrict__ spec) {
   extern __shared__ float4 smem[];
   const int n = ax.n, nh = n / 2 + 1;
   float4 *a = smem, *b = smem + n * kCols, *tw = smem + 2 * n * kCols;
   load_twiddles(tw, ax);
   const int64_t row0 = (int64_t)blockIdx.x * 2 * kCols;
-  for (int i = threadIdx.x; i < n * kCols; i += blockDim.x) {
-    const int c = i / n, x = i - c * n;
-    const int64_t r = row0 + 2 * c;
-    const float re = r < rows ? field[r * n + x] : 0.0f, im = r + 1 < rows ? field[(r + 1) * n + x] : 0.0f;
-    a[x * kCols + c] = make_float4(re, 0.0f, im, 0.0f);
-  }
+  // (the last stage stores into the buffer that it does not read)
+  float4* const out = ax.nfactors % 2 ? a : b;
+  transform<kOdd>(a, b, tw, ax,
+                  [&](int x, int c) {
+                    const int64_t r = row0 + 2 * c;
+                    return Cpx{{r < rows ? field[r * n + x] : 0.0f, 0.0f},
+                               {r + 1 < rows ? field[(r + 1) * n + x] : 0.0f, 0.0f}};
+                  },
+                  [&](int i, int c, const Cpx& v) { out[i * kCols + c] = pack(v); });
   __syncthreads();
-  a = transform<kOdd>(a, b, tw, ax);
   for (int i = threadIdx.x; i < nh * kCols; i += blockDim.x) {
-    const int c = i / nh, k = i - c * nh;
+    const int c = i % kCols, k = i / kCols;
     const int64_t r = row0 + 2 * c;
     if (r >= rows) continue;
-    const Cpx p = unpack(a[k * kCols + c]), q = unpack(a[(k == 0 ? 0 : n - k) * kCols + c]);
+    const Cpx p = unpack(out[k * kCols + c]), q = unpack(out[(k == 0 ? 0 : n - k) * kCols + c]);
     const auto half = [](Pair32 v) { return Pair32{0.5f * v.hi, 0.5f * v.lo}; };
     spec[r * nh + k] = pack(Cpx{half(padd(p.re, q.re)), half(psub(p.im, q.im))});
     if (r + 1 < rows) spec[(r + 1) * nh + k] = pack(Cpx{half(padd(p.im, q.im)), half(psub(q.re, p.re))});
@@ -206,37 +229,34 @@ __global__ void __launch_bounds__(256) k_spectrum_x(const __grid_constant__ Spec
 // Lines of n values `inner` apart: line l = (l / inner, l % inner) starts at (l / inner) n inner +
 // l % inner. In place, or |F|^2 (hi, lo) to `power`.
 template <int kOdd, bool kPower>
-__global__ void __launch_bounds__(256) k_spectrum_lines(const __grid_constant__ SpectrumAxis ax, float4* __restrict__ spec, uint32_t lines,
-                                                         FastDiv inner, float2* __restrict__ power,
+__global__ void __launch_bounds__(256) k_spectrum_lines(const __grid_constant__ SpectrumAxis ax, float4* __restrict__ spec,
+                                                         uint32_t lines, FastDiv inner, float2* __restrict__ power,
                                                          unsigned* __restrict__ range) {
   extern __shared__ float4 smem[];
   const int n = ax.n;
   float4 *a = smem, *b = smem + n * kCols, *tw = smem + 2 * n * kCols;
   load_twiddles(tw, ax);
   // (blockDim.x is a multiple of kCols: a thread stays with one line)
-  const int c = threadIdx.x % kCols;
-  const uint32_t l = blockIdx.x * (uint32_t)kCols + c;
+  const uint32_t l = blockIdx.x * (uint32_t)kCols + threadIdx.x % kCols;
   const uint32_t o = fastdiv(l, inner);
+  const bool mine = l < lines;
   const int64_t at = (int64_t)o * n * inner.d + (l - o * inner.d);
-  for (int i = threadIdx.x / kCols; i < n; i += blockDim.x / kCols)
-    a[i * kCols + c] = l < lines ? spec[at + (int64_t)i * inner.d] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-  __syncthreads();
-  a = transform<kOdd>(a, b, tw, ax);
   unsigned seen = 0u;
-  for (int i = threadIdx.x / kCols; i < n && l < lines; i += blockDim.x / kCols) {
-    const float4 v = a[i * kCols + c];
-    if (kPower) {
-      const Cpx f = unpack(v);
-      const Pair32 q = padd(pmul(f.re, f.re), pmul(f.im, f.im));
-      power[at + (int64_t)i * inner.d] = make_float2(q.hi, q.lo);
-      const float most = fmaxf(fabsf(v.x), fabsf(v.z));
-      // (a NaN is lost by fmaxf: its sum is not)
-      seen |= (v.x + v.z < 0x1p60f && v.x + v.z > -0x1p60f && most < 0x1p60f ? 0u : kSpectrumLarge) |
-              (most >= 0x1p-30f ? kSpectrumUsual : 0u) | (most > 0.0f ? kSpectrumNonzero : 0u);
-    } else {
-      spec[at + (int64_t)i * inner.d] = v;
-    }
-  }
+  transform<kOdd>(a, b, tw, ax,
+                  [&](int i, int) { return unpack(mine ? spec[at + (int64_t)i * inner.d] : make_float4(0.0f, 0.0f, 0.0f, 0.0f)); },
+                  [&](int i, int, const Cpx& f) {
+                    if (!mine) return;
+                    if (!kPower) {
+                      spec[at + (int64_t)i * inner.d] = pack(f);
+                      return;
+                    }
+                    const Pair32 q = padd(pmul(f.re, f.re), pmul(f.im, f.im));
+                    power[at + (int64_t)i * inner.d] = make_float2(q.hi, q.lo);
+                    const float x = f.re.hi, y = f.im.hi, most = fmaxf(fabsf(x), fabsf(y));
+                    // (a NaN is lost by fmaxf: its sum is not)
+                    seen |= (x + y < 0x1p60f && x + y > -0x1p60f && most < 0x1p60f ? 0u : kSpectrumLarge) |
+                            (most >= 0x1p-30f ? kSpectrumUsual : 0u) | (most > 0.0f ? kSpectrumNonzero : 0u);
+                  });
   if (kPower) {
     seen = __reduce_or_sync(0xffffffffu, seen);
     if ((threadIdx.x & 31) == 0 && (seen & ~*(volatile unsigned*)range)) atomicOr(range, seen);
