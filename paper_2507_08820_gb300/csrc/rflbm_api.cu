@@ -16,18 +16,10 @@
 #include "../../include/rflbm_testing.h"
 #include "rflbm_aux.h"
 #include "rflbm_diag.h"
+#include "rflbm_host.h"
 #include "rflbm_spectrum.h"
 
 using namespace rflbm_dev;
-
-// Results of the synchronous calls, page-locked host memory: the kernels write it in place, so
-// that a call ends with one synchronisation and no copy.
-struct HostResults {
-  int err;
-  double stats[kStatOutFields];
-  double modes[2 * kQ];
-  unsigned spectrum_range;
-};
 
 struct rflbm {
   rflbm_config_t cfg;
@@ -512,11 +504,8 @@ rflbm_t* rflbm_create_ex(const rflbm_config_t* cfg) {
   e = cudaMalloc((void**)&h->partials, sizeof(double) * ((size_t)h->stat_blocks * kStatOutFields + 1));
   if (e == cudaSuccess)
     e = cudaMemset(h->partials + (size_t)h->stat_blocks * kStatOutFields, 0, sizeof(double));
-  if (e == cudaSuccess) e = cudaHostAlloc((void**)&h->host, sizeof(HostResults), cudaHostAllocDefault);
-  if (e == cudaSuccess) {
-    std::memset(h->host, 0, sizeof(HostResults));
-    h->err = &h->host->err;
-  }
+  if (e == cudaSuccess) e = acquire_host_results(&h->host);
+  if (e == cudaSuccess) h->err = &h->host->err;
   if (e == cudaSuccess && h->slab) e = cudaEventCreateWithFlags(&h->faces_ready, cudaEventDisableTiming);
   if (e == cudaSuccess && h->slab) e = cudaEventCreateWithFlags(&h->exchanged, cudaEventDisableTiming);
   if (e != cudaSuccess) {
@@ -545,7 +534,7 @@ void rflbm_destroy(rflbm_t* h) {
     cudaFree(h->buf[1]);
   }
   cudaFree(h->partials);
-  cudaFreeHost(h->host);
+  release_host_results(h->host);
   cudaFreeHost(h->host_shells);
   cudaFree(h->diag_partials);
   cudaFree(h->diag_field);

@@ -29,6 +29,7 @@
 
 #include "../../include/rflbm.h"
 #include "rflbm_aux.h"
+#include "rflbm_host.h"
 #include "tma.cuh"
 
 namespace rflbm_dev {
@@ -516,12 +517,7 @@ struct rflbm_batch {
   int tile = 0;  // requested tile size (0: autotuned per row length, -1: by the order of preference)
   int ctas_per_sm = 1;
   unsigned long long* run = nullptr;  // device: first step of the current run, its buffer
-  // page-locked host memory that the kernels write in place: the results of the synchronous calls
-  struct HostResults {
-    int err;
-    double stats[kStatOutFields];
-  };
-  HostResults* results = nullptr;
+  HostResults* results = nullptr;  // what the kernels write for the synchronous calls
   int* err = nullptr;  // results->err
   double* partials = nullptr;
   int stat_blocks = 0;
@@ -963,11 +959,8 @@ rflbm_batch_t* rflbm_batch_create(const rflbm_replica_t* reps, int n, double rho
   if (rc == RFLBM_OK) {
     cudaError_t e = cudaMalloc((void**)&b->run, 2 * sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaMemset(b->run, 0, 2 * sizeof(unsigned long long));
-    if (e == cudaSuccess) e = cudaHostAlloc((void**)&b->results, sizeof(*b->results), cudaHostAllocDefault);
-    if (e == cudaSuccess) {
-      std::memset(b->results, 0, sizeof(*b->results));
-      b->err = &b->results->err;
-    }
+    if (e == cudaSuccess) e = acquire_host_results(&b->results);
+    if (e == cudaSuccess) b->err = &b->results->err;
     if (e != cudaSuccess) rc = bcuda(e, "allocating batch descriptors");
   }
   if (rc == RFLBM_OK) {
@@ -997,7 +990,7 @@ void rflbm_batch_destroy(rflbm_batch_t* b) {
   cudaFree(b->tile_rep);
   cudaFree(b->maps);
   cudaFree(b->run);
-  cudaFreeHost(b->results);
+  release_host_results(b->results);
   cudaFree(b->partials);
   cudaFree(b->staging);
   if (b->exec) cudaGraphExecDestroy(b->exec);
