@@ -79,19 +79,24 @@ typedef enum {
   RFLBM_PHI_RHO0 = 1       /* rho in Eq. 10 is the reference density rho0 */
 } rflbm_phi_rho;
 
-/* Step kernels. Both compute the same step; they differ in how the 27 neighbours are
- * fetched. The TMA kernel runs in row segments of 128, 192, 96, 64 or 32 sites: the first
+/* Step kernels. All compute the same step bit for bit; they differ in how the 27 neighbours are
+ * fetched. The TMA kernels run in row segments of 128, 192, 96, 64 or 32 sites: the first
  * that divides nx when nx is a multiple of 32; otherwise, when a row is a whole number of
  * 16-byte units (nx a multiple of 4 in float32, of 8 in 16-bit storage), the width whose
  * segments cover the row with the fewest idle threads per measured efficiency, the last
  * segment of each row ending past it, provided at least 77 % of the threads stay busy
- * (rflbm_step_path reports the width). On other boxes every choice runs the general kernel.
- * Some variants of the TMA kernel update two sites per thread with packed arithmetic
+ * (rflbm_step_path reports the width); or in flat tiles of 128 consecutive sites, whatever rows
+ * they lie in, on whole boxes of nx >= 16 where segments fit the rows badly (measured sizes: boxes
+ * of about 200,000 sites and more whose rows no width divides, or only 32 sites). The general
+ * kernel runs on every box: where the TMA kernels do not apply, and, with RFLBM_KERNEL_AUTO, on small
+ * boxes (with noise below about 112,000 sites, 190,000 where no width divides the rows), where
+ * a step lasts as long as its chain of latencies.
+ * Some variants of the TMA kernels update two sites per thread with packed arithmetic
  * (rflbm_step_sites_per_thread), bit for bit like the one-site forms. */
 typedef enum {
-  RFLBM_KERNEL_AUTO = 0,    /* TMA when the box allows it, else the general kernel */
-  RFLBM_KERNEL_GATHER = 1,  /* one thread per site, 27 addressed loads */
-  RFLBM_KERNEL_TMA = 2      /* one CTA per row segment, TMA tensor loads and stores */
+  RFLBM_KERNEL_AUTO = 0,    /* the fastest for the box (above) */
+  RFLBM_KERNEL_GATHER = 1,  /* the general kernel: one thread per site, 27 addressed loads */
+  RFLBM_KERNEL_TMA = 2      /* TMA tensor loads and stores when the box allows them */
 } rflbm_kernel;
 
 /* Streaming pattern (Eq. 8 carried out in memory).
@@ -245,15 +250,17 @@ int rflbm_synchronize(rflbm_t* h);
 int rflbm_get_dims(const rflbm_t* h, int* nx, int* ny, int* nz);
 int rflbm_launches_per_step(const rflbm_t* h);
 
-/* Step kernel the handle runs (an rflbm_kernel value other than AUTO); *width, if not
- * NULL, receives the row-segment width of the TMA kernels (0 for the general kernel). */
+/* Step kernel that the box's rows allow (an rflbm_kernel value other than AUTO): TMA when row
+ * segments cover them, and *width, if not NULL, receives the segment width; else the general
+ * kernel and 0. (Flat tiles and the general kernel on small boxes, see rflbm_kernel, change neither
+ * the report nor the values.) */
 int rflbm_step_path(const rflbm_t* h, int* width);
 
-/* Sites one thread of the kernel of the next step (rflbm_step(h, 1)) updates: 2 where the
+/* Sites one thread of the TMA kernel of the next step (rflbm_step(h, 1)) updates: 2 where the
  * TMA kernels run their two-site form (packed f32x2 arithmetic, one instruction for both
  * sites): Reg-FLBM with 16-bit storage and float32 without noise in either streaming
- * pattern, and the odd AA steps of float32 Reg-FLBM whose rows span several segments; else
- * 1. Both forms compute every site bit for bit alike; negative rflbm_status on an invalid
+ * pattern, and the odd AA steps of float32 Reg-FLBM whose rows span several segments (flat tiles:
+ * rows of an even number of sites); else 1. Both forms compute every site bit for bit alike; negative rflbm_status on an invalid
  * handle. */
 int rflbm_step_sites_per_thread(const rflbm_t* h);
 
@@ -266,11 +273,14 @@ int rflbm_step_sites_per_thread(const rflbm_t* h);
  *   square, for the 27 modes m_k = sum_i e_ki f_i of Table II (Eq. 5); 27 doubles each in
  *   host memory. Per-site values are formed in float32.
  * rflbm_structure_factor: for one field (rflbm_field, per site), F(k) = sum_x phi(x)
- *   exp(-i k.x) by a 3-D FFT (cuFFT), S(k) = |F(k)|^2 / N, summed over the spherical
+ *   exp(-i k.x) by a 3-D FFT (the library's, in sums of two float32 values with an error near
+ *   1e-14 of the norm, for edges up to 768 without a prime factor above 13 and fields whose
+ *   spectra have squares in the range of float32; else cuFFT in FP64), S(k) = |F(k)|^2 / N, summed
+ *   over the spherical
  *   shells n = round(|k| L / 2 pi), L = max(nx, ny, nz): s_sum[n] = sum of S over the
  *   wave vectors of shell n, count[n] = their number (n < nshell; both host arrays of
- *   nshell doubles; the k = 0 vector is in shell 0). Work buffers (two N-sized FP64 arrays
- *   and the FFT plan) are allocated on first use and kept by the handle.
+ *   nshell doubles; the k = 0 vector is in shell 0). Work buffers (an N-sized FP64 array, the
+ *   spectrum and the transform's tables or plan) are allocated on first use and kept by the handle.
  * rflbm_shell_count: the number of shells that covers every wave vector of the box. */
 typedef enum {
   RFLBM_FIELD_RHO = 0,  /* rho - rho0 */
