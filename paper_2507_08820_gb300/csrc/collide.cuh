@@ -347,19 +347,11 @@ __device__ __forceinline__ void collide_tile_bgk(V (&G)[3][3][3], const CollideP
     }
 }
 
-template <int kModel, bool kNoise, bool kGhostNeq, bool kPhiRho0, class V, class Noise, class OutWeight,
-          class Reload = KeepTile>
-__device__ __forceinline__ void collide_tile(V (&G)[3][3][3], const CollideParams& cp,
-                                          const Noise& noise, const OutWeight& outw,
-                                          const Reload& reload = Reload()) {
-  if (kModel == kModelBgk) {
-    collide_tile_bgk<kNoise, kPhiRho0>(G, cp, noise, outw, reload);
-    return;
-  }
-  // ---- 1. moments of order <= 2
-  V drho, jx, jy, jz, sxy, sxz, syz, axx, ayy, azz;
-  moments_order2(G, drho, jx, jy, jz, sxy, sxz, syz, axx, ayy, azz);
-
+// Reg-FLBM from the moments of order <= 2: the post-collision populations into G.
+template <bool kNoise, bool kGhostNeq, bool kPhiRho0, class V, class Noise, class OutWeight>
+__device__ __forceinline__ void collide_moments(V drho, V jx, V jy, V jz, V sxy, V sxz, V syz, V axx, V ayy, V azz,
+                                                V (&G)[3][3][3], const CollideParams& cp, const Noise& noise,
+                                                const OutWeight& outw) {
   // ---- 2. density, velocity and the scaled post-collision moments
   const V rho = vadd(splat<V>(cp.rho0), drho);
   const V inv_rho = vrcp(rho);
@@ -426,6 +418,21 @@ __device__ __forceinline__ void collide_tile(V (&G)[3][3][3], const CollideParam
   }
   inject_noise<kNoise, kPhiRho0>(M, rho, cp, noise);
   back_transform(M, G, outw);
+}
+
+template <int kModel, bool kNoise, bool kGhostNeq, bool kPhiRho0, class V, class Noise, class OutWeight,
+          class Reload = KeepTile>
+__device__ __forceinline__ void collide_tile(V (&G)[3][3][3], const CollideParams& cp,
+                                          const Noise& noise, const OutWeight& outw,
+                                          const Reload& reload = Reload()) {
+  if constexpr (kModel == kModelBgk) {
+    collide_tile_bgk<kNoise, kPhiRho0>(G, cp, noise, outw, reload);
+  } else {
+    // ---- 1. moments of order <= 2
+    V drho, jx, jy, jz, sxy, sxz, syz, axx, ayy, azz;
+    moments_order2(G, drho, jx, jy, jz, sxy, sxz, syz, axx, ayy, azz);
+    collide_moments<kNoise, kGhostNeq, kPhiRho0>(drho, jx, jy, jz, sxy, sxz, syz, axx, ayy, azz, G, cp, noise, outw);
+  }
 }
 
 // The collision of one site per thread with its normals drawn beforehand and the lattice

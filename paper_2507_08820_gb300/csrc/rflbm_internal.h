@@ -88,11 +88,6 @@ __device__ __forceinline__ Neighbours neighbours(uint32_t s, const Geometry& g) 
   return nb;
 }
 
-// Site that population i of site x is pulled from: x - c_i.
-__device__ __forceinline__ uint32_t pull_site(const Neighbours& nb, int i) {
-  return nb.X[cx_of(i) + 1] + nb.Y[cy_of(i) + 1] + nb.Z[cz_of(i) + 1];
-}
-
 // Element offsets of the 27 values g_i(s, t) of site s in a buffer of view g.view. The view is
 // resolved once per site (the natural view has the site itself in place of its neighbours, the
 // flipped one counts the planes down from the last), so that the offsets are sums without

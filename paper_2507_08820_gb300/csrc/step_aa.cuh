@@ -304,13 +304,16 @@ __global__ void __launch_bounds__(kW / 2) step_aa_even_pair(const __grid_constan
   }
 
   float2 G[3][3][3];
+  if constexpr (S::kScaled) {
+    collide_stored<kStore, kNoise>(
+        [&](int a, int b, int c, T (&v)[2]) { stored_pair(sm + (9 * b + 3 * c + a) * kW + 2 * t, true, v); }, p.ss, G, p.cp,
+        noise, ScaledWeight<kStore>{p.ss});
+  } else {
 #pragma unroll
-  for (int i = 0; i < kQ; ++i) {
-    float2 v = S::load2(sm + plane_of(i) * kW + 2 * t);
-    if (S::kScaled) v = kmul(p.ss.inv_scale[class_of(i)], v);
-    G[cx_of(i) + 1][cy_of(i) + 1][cz_of(i) + 1] = v;
+    for (int i = 0; i < kQ; ++i)
+      G[cx_of(i) + 1][cy_of(i) + 1][cz_of(i) + 1] = S::load2(sm + plane_of(i) * kW + 2 * t);
+    collide_tile<kModelReg, kNoise, false, false>(G, p.cp, noise, ScaledWeight<kStore>{p.ss});
   }
-  collide_tile<kModelReg, kNoise, false, false>(G, p.cp, noise, ScaledWeight<kStore>{p.ss});
 
   __syncthreads();  // all inputs are read: the tile can take the outputs
 #pragma unroll
@@ -394,15 +397,18 @@ __global__ void __launch_bounds__(kW / 2) step_aa_odd_pair(const __grid_constant
 
   float2 G[3][3][3];
   const T* mine = sm + kH + 2 * t;
+  const auto at = [&](int a, int b, int c) { return mine + (3 * b + c) * L::kGroup + (2 - a) * L::kSeg - (a - 1); };
+  if constexpr (S::kScaled) {
+    collide_stored<kStore, kNoise>([&](int a, int b, int c, T (&v)[2]) { stored_pair(at(a, b, c), a == 1, v); }, p.ss, G,
+                                   p.cp, noise, ScaledWeight<kStore>{p.ss});
+  } else {
 #pragma unroll
-  for (int i = 0; i < kQ; ++i) {
-    const int gi = 3 * (cy_of(i) + 1) + (cz_of(i) + 1);
-    const T* at = mine + gi * L::kGroup + (1 - cx_of(i)) * L::kSeg - cx_of(i);
-    float2 v = cx_of(i) == 0 ? S::load2(at) : S::load1x2(at);
-    if (S::kScaled) v = kmul(p.ss.inv_scale[class_of(i)], v);
-    G[cx_of(i) + 1][cy_of(i) + 1][cz_of(i) + 1] = v;
+    for (int i = 0; i < kQ; ++i) {
+      const int a = cx_of(i) + 1, b = cy_of(i) + 1, c = cz_of(i) + 1;
+      G[a][b][c] = a == 1 ? S::load2(at(a, b, c)) : S::load1x2(at(a, b, c));
+    }
+    collide_tile<kModelReg, kNoise, false, false>(G, p.cp, noise, ScaledWeight<kStore>{p.ss});
   }
-  collide_tile<kModelReg, kNoise, false, false>(G, p.cp, noise, ScaledWeight<kStore>{p.ss});
 
   if (kFullRow) {
     using O = AaRowOut<kStore, kW>;

@@ -78,6 +78,22 @@ struct Storage<kStoreF16> {
   static __device__ __forceinline__ void store2(T* p, float2 v) {
     *reinterpret_cast<__half2*>(p) = __float22half2_rn(v);
   }
+  // v + c, v - c and v r + c rounded once to float32 (sm_100-family mixed-precision instructions)
+  static __device__ __forceinline__ float add(T v, float c) {
+    float d;
+    asm("add.rn.f32.f16 %0, %1, %2;" : "=f"(d) : "h"(__half_as_ushort(v)), "f"(c));
+    return d;
+  }
+  static __device__ __forceinline__ float sub(T v, float c) {
+    float d;
+    asm("sub.rn.f32.f16 %0, %1, %2;" : "=f"(d) : "h"(__half_as_ushort(v)), "f"(c));
+    return d;
+  }
+  static __device__ __forceinline__ float fma(T v, T r, float c) {
+    float d;
+    asm("fma.rn.f32.f16 %0, %1, %2, %3;" : "=f"(d) : "h"(__half_as_ushort(v)), "h"(__half_as_ushort(r)), "f"(c));
+    return d;
+  }
   static __device__ __forceinline__ T pack(float v) { return __float2half_rn(v); }
   static __device__ __forceinline__ float to_float(T v) { return __half2float(v); }
   static constexpr bool kScaled = true;
@@ -101,6 +117,23 @@ struct Storage<kStoreBF16> {
   }
   static __device__ __forceinline__ void store2(T* p, float2 v) {
     *reinterpret_cast<__nv_bfloat162*>(p) = __float22bfloat162_rn(v);
+  }
+  static __device__ __forceinline__ float add(T v, float c) {
+    float d;
+    asm("add.rn.f32.bf16 %0, %1, %2;" : "=f"(d) : "h"(__bfloat16_as_ushort(v)), "f"(c));
+    return d;
+  }
+  static __device__ __forceinline__ float sub(T v, float c) {
+    float d;
+    asm("sub.rn.f32.bf16 %0, %1, %2;" : "=f"(d) : "h"(__bfloat16_as_ushort(v)), "f"(c));
+    return d;
+  }
+  static __device__ __forceinline__ float fma(T v, T r, float c) {
+    float d;
+    asm("fma.rn.f32.bf16 %0, %1, %2, %3;"
+        : "=f"(d)
+        : "h"(__bfloat16_as_ushort(v)), "h"(__bfloat16_as_ushort(r)), "f"(c));
+    return d;
   }
   static __device__ __forceinline__ T pack(float v) { return __float2bfloat16_rn(v); }
   static __device__ __forceinline__ float to_float(T v) { return __bfloat162float(v); }
