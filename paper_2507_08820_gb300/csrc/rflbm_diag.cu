@@ -4,6 +4,7 @@
 #include <cufft.h>
 
 #include "rflbm_diag.h"
+#include "tma.cuh"
 #include "wide.cuh"
 
 namespace rflbm_dev {
@@ -123,6 +124,7 @@ __global__ void __launch_bounds__(kDiagBlock) k_reduce_columns(const double* __r
                                  double* __restrict__ out, unsigned* range = nullptr,
                                  unsigned* range_out = nullptr) {
   __shared__ double sh[kDiagBlock / 32];
+  grid_dependency_wait();
   const int col = blockIdx.x;
   if (range && col == 0 && threadIdx.x == 0) {
     *range_out = *range;
@@ -149,6 +151,8 @@ template <int kStore, int kField, class Out>
 __global__ void __launch_bounds__(kDiagBlock) k_field(Geometry g, StoreScale ss,
                                                       const typename Storage<kStore>::T* __restrict__ src,
                                                       Out* __restrict__ out) {
+  grid_launch_dependents();
+  grid_dependency_wait();
   const int64_t s = (int64_t)blockIdx.x * kDiagBlock + threadIdx.x;
   if (s >= g.n) return;
   const PopSlots slots((uint32_t)s, g);
@@ -217,7 +221,9 @@ __global__ void __launch_bounds__(kDiagBlock) k_shell_bins(Geometry g, FastDiv d
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   for (int j = threadIdx.x; j < kWarps * nshell; j += kDiagBlock) bins[j] = 0.0;
   for (int j = threadIdx.x; j < nshell; j += kDiagBlock) counts[j] = 0u;
+  grid_launch_dependents();
   __syncthreads();
+  grid_dependency_wait();
   double* const mine = bins + (size_t)wid * nshell;
   const int nxh = g.nx / 2 + 1;
   const int64_t total = (int64_t)g.nz * g.ny * nxh;  // at most n
@@ -292,8 +298,8 @@ cudaError_t launch_mode_sums(const Geometry& g, const StoreScale& ss, int kind, 
     case kStoreBF16: k_mode_sums<kStoreBF16><<<(unsigned)blocks, kDiagBlock, 0, st>>>(g, ss, (const DT<kStoreBF16>*)src, partials); break;
     default: return cudaErrorInvalidValue;
   }
-  k_reduce_columns<<<2 * kQ, kDiagBlock, 0, st>>>(partials, blocks, 2 * kQ, out54, nullptr, nullptr);
-  return cudaGetLastError();
+  if (cudaError_t e = cudaGetLastError()) return e;
+  return launch_chained(&k_reduce_columns, 2u * kQ, kDiagBlock, 0, st, partials, blocks, 2 * kQ, out54, nullptr, nullptr);
 }
 
 template <int kStore, int kField, class Out>
@@ -304,8 +310,7 @@ static cudaError_t launch_field_at(const Geometry& g, const StoreScale& ss, cons
   } else {
     if (field != kField) return launch_field_at<kStore, kField + 1>(g, ss, src, field, out, st);
     const unsigned blocks = (unsigned)(((int64_t)g.n + kDiagBlock - 1) / kDiagBlock);
-    k_field<kStore, kField><<<blocks, kDiagBlock, 0, st>>>(g, ss, (const DT<kStore>*)src, out);
-    return cudaGetLastError();
+    return launch_chained(&k_field<kStore, kField, Out>, blocks, kDiagBlock, 0, st, g, ss, (const DT<kStore>*)src, out);
   }
 }
 
@@ -338,9 +343,11 @@ static cudaError_t launch_bins(const Geometry& g, const Entry* spec, int nshell,
         cudaFuncSetAttribute(k_shell_bins<Entry>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  k_shell_bins<<<blocks, kDiagBlock, smem, st>>>(g, make_fastdiv(g.nx / 2 + 1), make_fastdiv(g.ny), spec, nshell, partials);
-  k_reduce_columns<<<2 * nshell, kDiagBlock, 0, st>>>(partials, blocks, 2 * nshell, out, range, range_out);
-  return cudaGetLastError();
+  if (cudaError_t e = launch_chained(&k_shell_bins<Entry>, (unsigned)blocks, kDiagBlock, smem, st, g,
+                                     make_fastdiv(g.nx / 2 + 1), make_fastdiv(g.ny), spec, nshell, partials))
+    return e;
+  return launch_chained(&k_reduce_columns, 2u * nshell, kDiagBlock, 0, st, partials, (int64_t)blocks, 2 * nshell, out, range,
+                        range_out);
 }
 cudaError_t launch_shell_bins(const Geometry& g, const void* spec, int nshell, int blocks,
                               double* partials, double* out, cudaStream_t st) {

@@ -177,6 +177,24 @@ struct TmaMaps {
 
 constexpr int kStepBlock = 64;  // threads per block of the general kernel
 
+// Launches a kernel by programmatic dependent launch: it may start while the previous kernel of the
+// stream drains, and waits for it (griddepcontrol.wait) before it touches global memory.
+template <class... Params, class... Args>
+cudaError_t launch_chained(void (*kernel)(Params...), unsigned blocks, unsigned threads, size_t smem, cudaStream_t st,
+                           const Args&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, Params(args)...);
+}
+
 // Variant flags of the step kernel.
 struct StepVariant {
   int model;        // kModelReg / kModelBgk

@@ -17,6 +17,7 @@
 // three passes of 128^3 took 24 + 21 + 23 us with the tile loaded to and stored from shared memory,
 // and 16 + 16 + 17 us with the first stage loading and the last one storing in global memory.
 #include "rflbm_spectrum.h"
+#include "tma.cuh"
 #include "wide.cuh"
 
 #include <cmath>
@@ -203,7 +204,9 @@ __global__ void __launch_bounds__(256) k_spectrum_x(const __grid_constant__ Spec
   extern __shared__ float4 smem[];
   const int n = ax.n, nh = n / 2 + 1;
   float4 *a = smem, *b = smem + n * kCols, *tw = smem + 2 * n * kCols;
+  grid_launch_dependents();
   load_twiddles(tw, ax);
+  grid_dependency_wait();
   const int64_t row0 = (int64_t)blockIdx.x * 2 * kCols;
   // (the last stage stores into the buffer that it does not read)
   float4* const out = ax.nfactors % 2 ? a : b;
@@ -235,7 +238,9 @@ __global__ void __launch_bounds__(256) k_spectrum_lines(const __grid_constant__ 
   extern __shared__ float4 smem[];
   const int n = ax.n;
   float4 *a = smem, *b = smem + n * kCols, *tw = smem + 2 * n * kCols;
+  grid_launch_dependents();
   load_twiddles(tw, ax);
+  grid_dependency_wait();
   // (blockDim.x is a multiple of kCols: a thread stays with one line)
   const uint32_t l = blockIdx.x * (uint32_t)kCols + threadIdx.x % kCols;
   const uint32_t o = fastdiv(l, inner);
@@ -316,14 +321,14 @@ cudaError_t launch_power_spectrum(const Geometry& g, const SpectrumAxis (&ax)[3]
   const auto lines = [&](auto* kernel, const SpectrumAxis& a, uint32_t nlines, uint32_t inner) {
     const size_t smem = line_smem(a.n);
     if (cudaError_t e = allow_smem(kernel, smem)) return e;
-    kernel<<<(nlines + kCols - 1) / kCols, line_threads(a.n), smem, st>>>(a, s, nlines, make_fastdiv(inner), power, range);
-    return cudaGetLastError();
+    return launch_chained(kernel, (nlines + kCols - 1) / kCols, (unsigned)line_threads(a.n), smem, st, a, s, nlines,
+                          make_fastdiv(inner), power, range);
   };
   const auto first = [&](auto* kernel) {
     const size_t smem = line_smem(ax[0].n);
     if (cudaError_t e = allow_smem(kernel, smem)) return e;
-    kernel<<<(unsigned)((rows + 2 * kCols - 1) / (2 * kCols)), line_threads(ax[0].n), smem, st>>>(ax[0], field, rows, s);
-    return cudaGetLastError();
+    return launch_chained(kernel, (unsigned)((rows + 2 * kCols - 1) / (2 * kCols)), (unsigned)line_threads(ax[0].n), smem,
+                          st, ax[0], field, rows, s);
   };
   cudaError_t e = ax[0].odd == 0   ? first(&k_spectrum_x<0>)
                   : ax[0].odd == 1 ? first(&k_spectrum_x<1>)

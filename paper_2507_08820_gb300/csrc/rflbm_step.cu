@@ -97,16 +97,7 @@ __global__ void __launch_bounds__(kStepBlock) step_aa_gather(const StepParams p)
 }
 
 static cudaError_t launch_general(void (*kernel)(StepParams), const StepParams& p, cudaStream_t stream) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((p.nrows * p.geo.nx + kStepBlock - 1) / kStepBlock);
-  cfg.blockDim = dim3(kStepBlock);
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, p);
+  return launch_chained(kernel, (p.nrows * p.geo.nx + kStepBlock - 1) / kStepBlock, kStepBlock, 0, stream, p);
 }
 
 template <int kStore, bool kOdd, int kModel, bool kNoise>

@@ -579,17 +579,7 @@ __global__ void __launch_bounds__(kFlatW / 2) step_flat_aa_odd_pair(const __grid
 
 template <class Kernel, class... Args>
 cudaError_t launch_flat(Kernel* kernel, int threads, size_t smem, const StepParams& p, cudaStream_t st, const Args&... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((p.geo.n + kFlatW - 1) / kFlatW);
-  cfg.blockDim = dim3((unsigned)threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, args..., p);
+  return launch_chained(kernel, (p.geo.n + kFlatW - 1) / kFlatW, (unsigned)threads, smem, st, args..., p);
 }
 
 template <int kStore, int kModel, bool kNoise, bool kGhostNeq, bool kPhiRho0>
