@@ -113,7 +113,7 @@ def measured_peak():
 
 # the sources the ping-pong TMA step kernel is compiled from (its translation unit and
 # every header it includes)
-STEP_KERNEL_SOURCES = ("collide.cuh", "d3q27.cuh", "philox.cuh", "rflbm_internal.h",
+STEP_KERNEL_SOURCES = ("collide.cuh", "collide16.cuh", "d3q27.cuh", "philox.cuh", "rflbm_internal.h",
                        "rflbm_step_tma.cu", "rflbm_step_tma16.cu", "step_tma.cuh", "storage.cuh",
                        "tma.cuh")
 AA_KERNEL_SOURCES = STEP_KERNEL_SOURCES + ("step_aa.cuh", "rflbm_step_aa_f32.cu", "rflbm_step_aa_f16.cu",
