@@ -67,7 +67,7 @@ __device__ __noinline__ void init_site_fp64(const Geometry& g, uint32_t s, float
 // that is the FP64 result; a site with any population that they leave open is redone in FP64
 // (rest states and velocities near 1e-8, where g_i is lost in the roundings of f_i; one site in
 // thousands for flows). Bound by the 32 bytes read and 108 written per site (146 us at
-// 192^3): with 100 FP64 operations for every site 192^3 took 1254 us, so 380.
+// 192^3): 192^3 takes 380 us, and took 1254 us with 100 FP64 operations for every site.
 template <int kStore>
 __global__ void __launch_bounds__(kAuxBlock) k_init_field(Geometry g, float rho0, StoreScale ss, const double* __restrict__ rho,
                              const double* __restrict__ u, typename Storage<kStore>::T* __restrict__ dst) {
@@ -170,8 +170,8 @@ __global__ void k_init_thermal(Geometry g, float rho0, float kT, StoreScale ss, 
     }
 }
 
-// Import and export move 216 bytes per site (f32): with the rest populations formed by four FP64
-// products in every thread 128^3 float32 took 96 us in and 116 us out, with them given 65 us both.
+// Import and export move 216 bytes per site (f32): 128^3 float32 takes 65 us each way, and took
+// 96 us in and 116 us out with the rest populations formed by four FP64 products in every thread.
 // Import of public-layout populations (double: exact shift in FP64; float: in FP32).
 template <class Tin, int kStore>
 __global__ void k_set_populations(Geometry g, RestPops<Tin> rest, StoreScale ss, const Tin* __restrict__ f,
@@ -276,8 +276,9 @@ __device__ __noinline__ void moments_fp64(const Geometry& g, uint32_t s, const S
 // FP64 moments of every site: sums of 27 float32 values carried in 64-bit integers (fixed_sums),
 // packed into FP64 by integer operations, so that 15 FP64 operations per site are left (the
 // density and the three quotients) where plain FP64 takes 250. Bound by the 108 bytes read and
-// 80 written per site (196 us at 192^3; plain FP64 3224 us, so 337). Values outside the split's range (a population of 2^114 or more, or all
-// below 2^-66 and not zero; non-finite ones) go through FP64.
+// 80 written per site (196 us at 192^3; it takes 337 us, plain FP64 took 3224 us). Values outside the
+// split's range (a population of 2^114 or more, or all below 2^-66 and not zero; non-finite ones)
+// go through FP64.
 template <int kStore>
 __global__ void __launch_bounds__(kAuxBlock) k_moments(Geometry g, double rho0, StoreScale ss,
                           const typename Storage<kStore>::T* __restrict__ src,
@@ -358,7 +359,7 @@ __device__ __noinline__ float speed64(float x, float y, float z, float r) {
 // block to finish adds the rows in a fixed order into out. Bound by the 108 bytes read per
 // site. A site's sums are taken into FP64 once per thread (RunningSum), not once per site: with
 // 20 FP64 operations per site, and the final sum in a launch of its own, 128^3 float32 took
-// 375 + 7 us, so 65.
+// 375 + 7 us, and takes 61 us.
 constexpr int kStatSums = 4;  // drho, j
 template <int kStore>
 __global__ void __launch_bounds__(kAuxBlock, 4) k_stats(Geometry g, float rho0, StoreScale ss,
