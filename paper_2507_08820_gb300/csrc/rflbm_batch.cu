@@ -966,7 +966,7 @@ rflbm_batch_t* rflbm_batch_create(const rflbm_replica_t* reps, int n, double rho
   if (rc == RFLBM_OK) {
     int64_t nmax = 0;
     for (int r = 0; r < n; ++r) nmax = std::max<int64_t>(nmax, b->host[r].geo.n);
-    b->stat_blocks = std::max(1, (int)std::min<int64_t>(4 * (int64_t)b->num_sms, (nmax + 255) / 256));
+    b->stat_blocks = std::max(1, (int)std::min<int64_t>(3 * (int64_t)b->num_sms, (nmax + 255) / 256));
     cudaError_t e = cudaMalloc((void**)&b->partials, sizeof(double) * ((size_t)b->stat_blocks * kStatOutFields + 1));
     if (e == cudaSuccess)
       e = cudaMemset(b->partials + (size_t)b->stat_blocks * kStatOutFields, 0, sizeof(double));
