@@ -304,7 +304,7 @@ __global__ void __launch_bounds__(kAuxBlock) k_moments(Geometry g, double rho0, 
   }
   long long t[10];
   fixed_sums(G, E, t);
-  const int k = (int)E - 182;
+  const int k = (int)E - 179;  // units of 2^(e - 53)
   if (rho || u) {
     const double r = rho0 + scaled_double(t[0], k);
     if (rho) rho[s] = r;

@@ -135,19 +135,20 @@ __device__ __forceinline__ void raw_sums(const float (&G)[3][3][3], float (&m)[1
   m[9] = __fsub_rn(T01[2], T01[0]);
 }
 
-// The same sums as integers in units of 2^(e - 56), where e is the least exponent with every
-// |g| < 2^e: each g is split on the grids 2^(e - 18) and 2^(e - 37); the sums of either part
-// are exact in float32 (27 2^18 units at most), and so is the remainder's to 2^(e - 53). An FP64
-// accumulation of the 27 terms keeps 2^(e - 50) or so. E = e + 126 (the exponent field of the
-// largest |g|), 60 <= E <= 240. G is used up.
+// The same sums as integers in units of 2^(e - 53), where e is the least exponent with every
+// |g| < 2^e: each g is split on the grids 2^(e - 17) and 2^(e - 35), so that in every part a g is at most
+// 2^17 of its units and a sum of 27 at most 27 2^17 < 2^22. The sums of the first two parts are exact in
+// float32, and so is the remainder's to 2^(e - 53); adding 1.5 2^23 leaves such an integer in the low bits, which holds
+// up to 2^22 only. An FP64 accumulation of the 27 terms keeps 2^(e - 50) or so. E = e + 126 (the
+// exponent field of the largest |g|), 60 <= E <= 240. G is used up.
 __device__ __forceinline__ void fixed_sums(float (&G)[3][3][3], uint32_t E, long long (&t)[10]) {
-  const float half23 = 12582912.0f;  // 1.5 2^23: adding it leaves the integer in the low bits
+  const float half23 = 12582912.0f;  // 1.5 2^23
   float m[10];
 #pragma unroll
   for (int part = 0; part < 3; ++part) {
-    const uint32_t down = part == 0 ? 271u : (part == 1 ? 290u : 309u);  // 1 / unit
+    const uint32_t down = part == 0 ? 270u : (part == 1 ? 288u : 306u);  // 1 / unit
     if (part < 2) {
-      const float grid = __uint_as_float(((part == 0 ? E + 6u : E - 13u) << 23) | 0x400000u);
+      const float grid = __uint_as_float(((part == 0 ? E + 7u : E - 11u) << 23) | 0x400000u);  // 1.5 2^23 units
       float H[3][3][3];
 #pragma unroll
       for (int a = 0; a < 3; ++a)
@@ -167,7 +168,7 @@ __device__ __forceinline__ void fixed_sums(float (&G)[3][3][3], uint32_t E, long
     for (int k = 0; k < 10; ++k) {
       const int n = __float_as_int(__fmaf_rn(m[k], scale, half23)) - __float_as_int(half23);
       if (part == 0) t[k] = n;
-      else t[k] = t[k] * 524288 + n;
+      else t[k] = t[k] * 262144 + n;
     }
   }
 }

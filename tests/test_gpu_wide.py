@@ -170,3 +170,36 @@ def test_structure_factor_of_a_fluid_at_rest_is_zero(R):
     s, count = R.rflbm_structure_factor(box.h, 0)
     box.close()
     assert not s.any() and count.sum() == 24 * 10 * 9
+
+
+def _sites_of_sums():
+    """Populations (27, n) whose sums come near the bound of their terms: all equal, of either sign, within 30 % of each
+    other, equal where c_x != 0, w_i times one density deviation, and equal values far below one that sets the scale,
+    with mantissas near all ones (each part of a split is then near its largest, with one sign)."""
+    g = np.random.default_rng(17)
+    one = np.ones((27, 1))
+    cx = o.velocities()[:, 0][:, None]
+    full = 1.0 - 2.0 ** -22
+    blocks = [s * v * one for s in (1.0, -1.0) for v in (0.1, 0.12, 0.5, full)]
+    blocks += [s * (0.05 * (1.0 + 0.3 * g.uniform(-1.0, 1.0, (27, 400)))) for s in (1.0, -1.0)]
+    blocks += [s * v * (cx != 0) for s in (1.0, -1.0) for v in (0.12, full)]
+    blocks += [o.weights()[:, None] * g.uniform(-0.1, 0.1, (1, 2000))]
+    low = np.repeat(full * 2.0 ** -np.arange(64)[None, :], 27, axis=0)
+    low[26] = 0.99
+    return np.float64(np.float32(np.concatenate(blocks + [low, -low], axis=1)))
+
+
+@pytest.mark.parametrize("scale", [2.0 ** -40, 1.0, 2.0 ** 90])
+def test_moments_of_sums_near_the_bound_of_their_terms(R, scale):
+    """Against FP64 sums at the tolerance of test_moments_match_fp64_sums, in both views of a site."""
+    f = scale * _sites_of_sums()
+    for pattern in (0, 1):
+        box = R.Box(f.shape[1], 1, 1, tau=0.8, rho0=1e-30, pattern=pattern)
+        R.rflbm_set_populations(box.h, np.ascontiguousarray(f))
+        got = box.populations()
+        rho, _, pi = box.macroscopic()
+        box.close()
+        wrho, _, wpi = o.macroscopic(got)
+        s = np.abs(got).sum(axis=0) + 1e-30
+        assert np.all(np.abs(rho - wrho) <= 64 * EPS * s)
+        assert np.all(np.abs(pi - wpi) <= 64 * EPS * s)
