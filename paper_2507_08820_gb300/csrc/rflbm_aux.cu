@@ -37,13 +37,16 @@ static RestPops<Tio> rest_pops(float rho0) {
   return r;
 }
 
-// delta = psi(c, u) / w_c - 1 for c = -1, 0, +1: 3 u^2 -+ 3 u, -3 u^2 / 2.
-__device__ __forceinline__ void psi_excess(Pair32 u, Pair32 (&d)[3]) {
+// delta = psi(c, u) / w_c - 1 for c = -1, 0, +1: 3 u^2 -+ 3 u, -3 u^2 / 2. size: the sum of the terms'
+// magnitudes, which the errors of d are relative to (near |u| = 1 the terms of c = -+1 cancel).
+__device__ __forceinline__ void psi_excess(Pair32 u, Pair32 (&d)[3], float (&size)[3]) {
   const Pair32 q = pmul(u, u);
   const Pair32 q3 = pmul(Pair32{3.0f, 0.0f}, q), u3 = pmul(Pair32{3.0f, 0.0f}, u);
   d[0] = padd(q3, Pair32{-u3.hi, -u3.lo});
   d[1] = pmul(Pair32{-1.5f, 0.0f}, q);
   d[2] = padd(q3, u3);
+  size[0] = size[2] = __fadd_rn(q3.hi, fabsf(u3.hi));
+  size[1] = fabsf(d[1].hi);
 }
 
 // g_i = r psi(c_x, u_x) psi(c_y, u_y) psi(c_z, u_z) - w_i rho0 of one site in FP64.
@@ -61,13 +64,14 @@ __device__ __noinline__ void init_site_fp64(const Geometry& g, uint32_t s, float
 
 // The same for every site, scattered to the view's slots. With psi(c, u) = w_c (1 + delta_c),
 // g_i / w_i = Q_ab + (rho0 + Q_ab) delta_c where Q_ab = r D_ab + (r - rho0) and 1 + D_ab =
-// (1 + delta_a)(1 + delta_b): no difference of nearly equal numbers is left, so sums of two
-// float32 values carry it to 2^-43 of its terms, and FP64 differs from it by no more than its own
-// dozen roundings of f_i. Where every value within these errors rounds to one float32 value,
-// that is the FP64 result; a site with any population that they leave open is redone in FP64
-// (rest states and velocities near 1e-8, where g_i is lost in the roundings of f_i; one site in
-// thousands for flows). Bound by the 32 bytes read and 108 written per site (146 us at
-// 192^3): 192^3 takes 380 us, and took 1254 us with 100 FP64 operations for every site.
+// (1 + delta_a)(1 + delta_b): the rest value is no difference any more, so sums of two float32 values
+// carry it to 2^-43 of the magnitudes of its terms, and FP64 differs from it by no more than its own dozen
+// roundings of f_i. Where every value within these errors rounds to one float32 value, that is
+// the FP64 result; a site with any population that they leave open is redone in FP64 (one site in
+// thousands for flows with velocities of a percent; most below 1e-6, where g_i is lost in the roundings of
+// f_i, and a warp with one such site takes as long as one of them). Bound by the 32 bytes read and
+// 108 written per site (146 us at 192^3): 192^3 takes 346 us with velocities of 2 %, 1228 us at rest or with
+// velocities up to 1e-4, and took 1255 us with 100 FP64 operations for every site.
 template <int kStore>
 __global__ void __launch_bounds__(kAuxBlock) k_init_field(Geometry g, float rho0, StoreScale ss, const double* __restrict__ rho,
                              const double* __restrict__ u, typename Storage<kStore>::T* __restrict__ dst) {
@@ -83,15 +87,16 @@ __global__ void __launch_bounds__(kAuxBlock) k_init_field(Geometry g, float rho0
     const PopSlots slots(site_of(s), g);
     const Pair32 R = pair_of(r), dR = pair_of(dr);
     Pair32 dx[3], dy[3], dz[3];
-    psi_excess(pair_of(ux), dx);
-    psi_excess(pair_of(uy), dy);
-    psi_excess(pair_of(uz), dz);
+    float tx[3], ty[3], tz[3];
+    psi_excess(pair_of(ux), dx, tx);
+    psi_excess(pair_of(uy), dy, ty);
+    psi_excess(pair_of(uz), dz, tz);
     const float own = fmaf(0x1p-43f, fabsf(dR.hi), 0x1p-48f * (fabsf(R.hi) + rho0));
 #pragma unroll
     for (int a = 0; a < 3; ++a)
 #pragma unroll
       for (int b = 0; b < 3; ++b) {
-        const float Aab = fmaf(fabsf(dx[a].hi), fabsf(dy[b].hi), fabsf(dx[a].hi) + fabsf(dy[b].hi));
+        const float Aab = fmaf(tx[a], ty[b], tx[a] + ty[b]);
         const Pair32 D = padd(padd(dx[a], dy[b]), pmul(dx[a], dy[b]));
         const Pair32 Q = padd(pmul(R, D), dR);
         const Pair32 P = padd(Pair32{rho0, 0.0f}, Q);
@@ -102,7 +107,7 @@ __global__ void __launch_bounds__(kAuxBlock) k_init_field(Geometry g, float rho0
           const int cls = class_at(a, b, c);
           const Pair32 W{(float)w[cls], (float)(w[cls] - (double)(float)w[cls])};
           const Pair32 v = pmul(W, padd(Q, pmul(P, dz[c])));
-          const float A = fmaf(fabsf(dz[c].hi), 1.0f + Aab, Aab);  // over |f_i / w_i r - 1| without cancellation
+          const float A = fmaf(tz[c], 1.0f + Aab, Aab);  // over the terms of f_i / w_i r - 1
           const float err = W.hi * fmaf(fabsf(R.hi) * A, 0x1.1p-43f, own);
           const float lo = __fadd_rn(v.hi, __fsub_rn(v.lo, err));
           open = open || !(lo == __fadd_rn(v.hi, __fadd_rn(v.lo, err)));

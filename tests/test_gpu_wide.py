@@ -203,3 +203,31 @@ def test_moments_of_sums_near_the_bound_of_their_terms(R, scale):
         s = np.abs(got).sum(axis=0) + 1e-30
         assert np.all(np.abs(rho - wrho) <= 64 * EPS * s)
         assert np.all(np.abs(pi - wpi) <= 64 * EPS * s)
+
+
+@pytest.mark.parametrize("others", [0.0, 0.1])
+def test_initial_fields_where_a_velocity_term_cancels(R, others):
+    """Near |u| = 1 the factor 1 - 3 |u| + 3 u^2 of a population is near 1 with large terms. g is the float32
+    nearest to f - w rho0 up to the FP64 roundings of f: three of each of the three factors' terms, and four of
+    their product with the density and its difference from the rest value."""
+    g = np.random.default_rng(23)
+    n = 6000
+    near = lambda: g.choice([-1.0, 1.0], n) * (1.0 + g.choice([-1.0, 1.0], n) * 2.0 ** -g.uniform(1, 50, n))  # noqa: E731
+    u = np.stack([near(), others * g.uniform(-1, 1, n), others * near()])
+    for k in range(1, 3):  # every axis
+        u[:, k::3] = np.roll(u[:, k::3], k, axis=0)
+    rho = np.ones(n)
+    box = R.Box(n, 1, 1, tau=0.8)
+    R.rflbm_init_field(box.h, rho, np.ascontiguousarray(u))
+    got = box.populations()
+    box.close()
+    w = o.weights()[:, None].astype(np.longdouble)
+    v = u.astype(np.longdouble)
+    f, size = w * rho, w * rho
+    for a, c in enumerate(o.velocities().T):
+        c = c[:, None]
+        f = f * np.where(c == 0, 1 - 1.5 * v[a] ** 2, 1 + 3 * c * v[a] + 3 * v[a] ** 2)
+        size = size * (1 + 3 * np.abs(v[a]) + 3 * v[a] ** 2)
+    stored = (got.astype(np.longdouble) - w).astype(np.float32)  # (the export rounds f to FP64)
+    tol = 0.5000001 * np.spacing(np.abs(stored)).astype(float) + 16 * EPS * size
+    assert np.all(np.abs(stored.astype(np.longdouble) - (f - w)) <= tol)
