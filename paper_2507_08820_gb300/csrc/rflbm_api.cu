@@ -245,6 +245,15 @@ int check_ready(const rflbm* h) {
   return RFLBM_OK;
 }
 
+// Clears and copies on the legacy stream are complete for work that follows on `st`: a blocking
+// stream waits for them by itself, a non-blocking one does not (and one under capture cannot be made to).
+cudaError_t settle_for(cudaStream_t st) {
+  if (st == nullptr || st == cudaStreamLegacy || st == cudaStreamPerThread) return cudaSuccess;
+  unsigned flags = 0;
+  if (cudaError_t e = cudaStreamGetFlags(st, &flags)) return e;
+  return flags & cudaStreamNonBlocking ? cudaStreamSynchronize(cudaStreamLegacy) : cudaSuccess;
+}
+
 int sync(rflbm* h, const char* what) {
   RFLBM_CUDA(cudaStreamSynchronize(h->stream), what);
   volatile int* const flag = h->err;
@@ -508,6 +517,7 @@ rflbm_t* rflbm_create_ex(const rflbm_config_t* cfg) {
   if (e == cudaSuccess) h->err = &h->host->err;
   if (e == cudaSuccess && h->slab) e = cudaEventCreateWithFlags(&h->faces_ready, cudaEventDisableTiming);
   if (e == cudaSuccess && h->slab) e = cudaEventCreateWithFlags(&h->exchanged, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = settle_for(h->stream);
   if (e != cudaSuccess) {
     cuda_fail(e, "allocating the reduction scratch");
     rflbm_destroy(h);
@@ -878,6 +888,7 @@ int rflbm_structure_factor(rflbm_t* h, int field, int nshell, double* s_sum, dou
       const size_t bytes = sizeof(float) * table.size();
       if (!h->twiddles) RFLBM_CUDA(cudaMalloc((void**)&h->twiddles, bytes), "allocating the twiddle factors");
       RFLBM_CUDA(cudaMemcpy(h->twiddles, table.data(), bytes, cudaMemcpyHostToDevice), "copying the twiddle factors");
+      RFLBM_CUDA(settle_for(h->stream), "waiting for the twiddle factors");
       int at = 0;
       for (int a = 0; a < 3; at += edge[a++]) h->axes[a].twiddles = h->twiddles + at;
       h->spectrum_range = reinterpret_cast<unsigned*>(h->twiddles + at);

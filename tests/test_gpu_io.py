@@ -48,3 +48,34 @@ def test_float32_import_and_export(R, shape, where, pattern):
     box.close()
     assert np.array_equal(out_pinned.numpy(), out_pageable)
     assert np.allclose(out_pageable, f32, rtol=2.5e-7, atol=0)
+
+
+@pytest.mark.parametrize("pattern", [0, 1])
+def test_a_new_handle_is_ready_on_a_non_blocking_stream(R, pattern):
+    """A handle's clears and tables go through the legacy stream. While that is busy, a handle of a non-blocking
+    stream still reads and writes its own state."""
+    import torch
+    shape = (24, 10, 9)
+    n = int(np.prod(shape))
+    f = o.rest_state(n) + W.population_perturbation(n, 3, 1e-3)
+    ref = R.Box(*shape, tau=0.8, pattern=pattern)
+    R.rflbm_set_populations(ref.h, np.ascontiguousarray(f))
+    want = (ref.populations(), R.rflbm_stats(ref.h)[0], R.rflbm_structure_factor(ref.h, 1))
+    ref.close()
+    busy = torch.empty(1 << 28, dtype=torch.float32, device="cuda")
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    for _ in range(5):
+        for _ in range(40):  # some 8 ms of fills on the legacy stream
+            busy.fill_(1.0)
+        box = R.Box(*shape, tau=0.8, pattern=pattern, stream=side.cuda_stream)
+        R.rflbm_set_populations(box.h, np.ascontiguousarray(f))
+        st, status = R.rflbm_stats(box.h)
+        for _ in range(40):
+            busy.fill_(2.0)
+        s, c = R.rflbm_structure_factor(box.h, 1)
+        got = box.populations()
+        box.close()
+        assert np.array_equal(got, want[0]) and status == R.RFLBM_OK
+        assert (st.mass, list(st.momentum), st.max_speed) == (want[1].mass, list(want[1].momentum), want[1].max_speed)
+        assert np.array_equal(s, want[2][0]) and np.array_equal(c, want[2][1])
