@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(kTile, kRows ? 65536 / (kTile * 56) : 0)
 #pragma unroll
     for (int i = 0; i < kQ; ++i)
       G[cx_of(i) + 1][cy_of(i) + 1][cz_of(i) + 1] =
-          S::load(__ldg(src + s + pull_delta(d, i) + plane_of(i) * rep.geo.ps), class_of(i), rep.ss);
+          S::load(src[s + pull_delta(d, i) + plane_of(i) * rep.geo.ps], class_of(i), rep.ss);
     if (rep.noise)
       collide_site<kModelReg, true, false, false>(G, rep.cp, noise);
     else

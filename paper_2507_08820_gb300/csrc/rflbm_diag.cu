@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(kDiagBlock, 2) k_mode_sums(Geometry g, StoreSc
 
 // Column sums of a row-major array in a fixed order: a block per column, thread t adds rows
 // t, t + 256, ..., then a fixed tree.
-__global__ void __launch_bounds__(kDiagBlock) k_reduce_columns(const double* __restrict__ partials, int64_t rows, int cols,
+__global__ void __launch_bounds__(kDiagBlock) k_reduce_columns(const double* partials, int64_t rows, int cols,
                                  double* __restrict__ out, unsigned* range = nullptr,
                                  unsigned* range_out = nullptr) {
   __shared__ double sh[kDiagBlock / 32];
@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(kDiagBlock) k_reduce_columns(const double* __r
 // float32); bound by the 108 bytes read and 8 written per site.
 template <int kStore, int kField, class Out>
 __global__ void __launch_bounds__(kDiagBlock) k_field(Geometry g, StoreScale ss,
-                                                      const typename Storage<kStore>::T* __restrict__ src,
+                                                      const typename Storage<kStore>::T* src,
                                                       Out* __restrict__ out) {
   grid_launch_dependents();
   grid_dependency_wait();
@@ -216,7 +216,7 @@ __device__ __forceinline__ double fp64_of(Pair32 v) { return (double)v.hi + (dou
 // grid's, in one wave.)
 template <class Entry>
 __global__ void __launch_bounds__(kDiagBlock, 4) k_shell_bins(Geometry g, FastDiv div_nxh, FastDiv div_nyh,
-                                                           const Entry* __restrict__ spec, int nshell,
+                                                           const Entry* spec, int nshell,
                                                            double* __restrict__ partials) {
   constexpr int kWarps = kDiagBlock / 32;
   extern __shared__ double bins[];  // [kWarps][nshell] sums, then [nshell] counts

@@ -199,7 +199,7 @@ __device__ __forceinline__ void load_twiddles(float4* tw, const SpectrumAxis& ax
 // line p; their half spectra to spec[row][kx], kx <= n / 2.
 template <int kOdd>
 __global__ void __launch_bounds__(256) k_spectrum_x(const __grid_constant__ SpectrumAxis ax,
-                                                     const float* __restrict__ field, int64_t rows,
+                                                     const float* field, int64_t rows,
                                                      float4* __restrict__ spec) {
   extern __shared__ float4 smem[];
   const int n = ax.n, nh = n / 2 + 1;
@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(256) k_spectrum_x(const __grid_constant__ Spec
 // Lines of n values `inner` apart: line l = (l / inner, l % inner) starts at (l / inner) n inner +
 // l % inner. In place, or |F|^2 (hi, lo) to `power`.
 template <int kOdd, bool kPower>
-__global__ void __launch_bounds__(256) k_spectrum_lines(const __grid_constant__ SpectrumAxis ax, float4* __restrict__ spec,
+__global__ void __launch_bounds__(256) k_spectrum_lines(const __grid_constant__ SpectrumAxis ax, float4* spec,
                                                          uint32_t lines, FastDiv inner, float2* __restrict__ power,
                                                          unsigned* __restrict__ range) {
   extern __shared__ float4 smem[];

@@ -34,22 +34,35 @@ __global__ void __launch_bounds__(kStepBlock) step_pull(const StepParams p) {
     site_noise_part<0, 6>(s + p.geo.site0, p.step, p.replica, p.rk, noise);
     if (!normals_formed<24>(noise)) return;
   }
-  grid_dependency_wait();
+  // the nine source rows' addresses are formed before the wait too (behind it they are part of every step's
+  // chain: 32^3 float32 4.0 us per step, 3.6 so; all 27 addresses 4.2)
   const PullDeltas d = pull_deltas(s, p.geo);
   const int64_t sb = s + (int64_t)p.geo.zlo * p.geo.nxy;
-  const T* __restrict__ src = static_cast<const T*>(p.src) + sb;
+  const T* row[3][3];
+#pragma unroll
+  for (int b = 0; b < 3; ++b)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      row[b][c] = static_cast<const T*>(p.src) + sb + (d.DY[b] + d.DZ[c]) + 3 * (3 * b + c) * p.geo.ps;
+      asm volatile("" : "+l"(row[b][c]));
+    }
+  int32_t right = d.DX[0], left = d.DX[2];
+  asm volatile("" : "+r"(right), "+r"(left));
+  grid_dependency_wait();
 
+  // pre-collision populations: g_i(x, t) pulled from x - c_i, by plain loads: the previous step wrote these
+  // values while this kernel was already running, and data read through the read-only path has to stay unchanged
+  // for a kernel's lifetime
   float G[3][3][3];
 #pragma unroll
   for (int i = 0; i < kQ; ++i) {
-    // per-thread neighbour pointer plus the plane offset i * ps (uniform across the grid)
-    G[cx_of(i) + 1][cy_of(i) + 1][cz_of(i) + 1] =
-        S::load(__ldg((src + pull_delta(d, i)) + plane_of(i) * p.geo.ps), class_of(i), p.ss);
+    const int a = cx_of(i) + 1, b = cy_of(i) + 1, c = cz_of(i) + 1;
+    G[a][b][c] = S::load(row[b][c][a * p.geo.ps + (a == 1 ? 0 : a == 0 ? right : left)], class_of(i), p.ss);
   }
 
   collide_site<kModel, kNoise, kGhostNeq, kPhiRho0>(G, p.cp, noise);
 
-  T* __restrict__ dst = static_cast<T*>(p.dst) + sb;
+  T* dst = static_cast<T*>(p.dst) + sb;
 #pragma unroll
   for (int i = 0; i < kQ; ++i)
     dst[plane_of(i) * p.geo.ps] = S::store(G[cx_of(i) + 1][cy_of(i) + 1][cz_of(i) + 1], class_of(i), p.ss);
