@@ -89,7 +89,7 @@ typedef enum {
  * they lie in, on whole boxes of nx >= 16 where segments fit the rows badly (measured sizes: boxes
  * of about 200,000 sites and more whose rows no width divides, or only 32 sites). The general
  * kernel runs on every box: where the TMA kernels do not apply, and, with RFLBM_KERNEL_AUTO, on small
- * boxes (with noise below about 112,000 sites, 190,000 where no width divides the rows), where
+ * boxes (with noise from 4096 to about 112,000 sites, 190,000 where no width divides the rows), where
  * a step lasts as long as its chain of latencies.
  * Some variants of the TMA kernels update two sites per thread with packed arithmetic
  * (rflbm_step_sites_per_thread), bit for bit like the one-site forms. */

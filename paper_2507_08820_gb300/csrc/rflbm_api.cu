@@ -283,14 +283,16 @@ bool setup_flat(rflbm* h) {
 
 // Whole boxes of the automatic choice whose TMA steps are slower than the general kernel's for
 // their latency alone. Microseconds per step, TMA against general: with noise 32^3 float32 6.5 and
-// 4.3, AA 5.3 and 2.9, float16 7.9 and 5.0; 96x32x32 5.6 and 4.7, float16 8.1 and 5.3;
-// 128x32x32 (131,072 sites) 6.3 and 6.6. Without noise float32 32^3 6.2 and 5.1, 96x32x32 6.1 and
-// 6.0; 16-bit 32^3 5.6 and 6.0.
-// Rows that no segment width divides: 56^3 (ragged segments) 9.2 and 8.5, without noise 9.6 and 6.3;
-// 80^3 without noise 17.9 and 15.8. Ragged segments of 128 sites and more without noise in 16-bit
-// storage are like whole ones (128x32x32 5.2 and 7.0).
+// 3.6, AA 5.1 and 2.9, float16 7.8 and 3.4; 96x32x32 6.3 and 4.9, float16 8.0 and 5.3;
+// 128x32x32 (131,072 sites) 6.1 and 5.3, float16 8.2 and 5.8, BGK 6.0 and 6.0. Without noise float32 32^3 6.1
+// and 3.9, 96x32x32 6.2 and 5.0; 16-bit 32^3 5.5 and 5.2, 96x32x32 4.9 and 6.1.
+// Rows that no segment width divides: 56^3 (ragged segments) 9.3 and 7.5, without noise 10.5 and 5.5;
+// 80^3 20.0 (flat tiles) and 22.0, without noise 15.0 and 15.6. Ragged segments of 128 sites and more without noise in
+// 16-bit storage are like whole ones (128x32x32 5.1 and 6.3).
+// Boxes below 4096 sites run what their rows allow: both kernels are near the rate of launches there
+// (64x6x5 float32 2.3 and 2.1, float16 3.3 and 2.0), and the choice follows the rows alone.
 bool general_pays(const rflbm* h) {
-  if (h->slab || h->cfg.kernel != RFLBM_KERNEL_AUTO) return false;
+  if (h->slab || h->cfg.kernel != RFLBM_KERNEL_AUTO || h->geo.n < 4096u) return false;
   const bool noise = h->variant.noise, f32 = h->variant.storage == kStoreF32;
   if (tma_segment_width(h->geo.nx) == 0 && !noise && !f32 && tma_ragged_width(h->geo.nx, 2) >= 128) return false;
   if (tma_segment_width(h->geo.nx) == 0) return h->geo.n < (noise ? 190000u : (f32 ? 450000u : 230000u));
@@ -631,12 +633,10 @@ cudaError_t launch_rows(rflbm* h, StepParams& p, uint32_t row0, uint32_t nrows, 
   p.nrows = nrows;
   p.row_split = split < nrows ? split : nrows;
   p.row_gap = gap;
-  // (the testing hook is about the TMA kernels' waits)
-  const bool general = h->small && !h->test_extra_tx;
   if (h->aa) {
     p.src = p.dst = h->buf[0];
     const bool odd = h->phase != 0;
-    if (general) return launch_step_aa_gather(p, h->variant, odd, h->stream);
+    if (h->small) return launch_step_aa_gather(p, h->variant, odd, h->stream);
     if (h->flat) {
       const TmaMaps m{&h->load_map[0], &h->store_map[0], 0};
       return launch_step_flat_aa(m, p, h->variant, odd, h->stream);
@@ -649,7 +649,7 @@ cudaError_t launch_rows(rflbm* h, StepParams& p, uint32_t row0, uint32_t nrows, 
   }
   p.src = h->buf[h->cur];
   p.dst = h->buf[1 - h->cur];
-  if (general) return launch_step_gather(p, h->variant, h->stream);
+  if (h->small) return launch_step_gather(p, h->variant, h->stream);
   if (h->flat) {
     const TmaMaps m{&h->load_map[h->cur], &h->store_map[1 - h->cur], 0};
     return launch_step_flat(m, p, h->variant, h->stream);
