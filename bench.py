@@ -116,6 +116,8 @@ def measured_peak():
 STEP_KERNEL_SOURCES = ("collide.cuh", "collide16.cuh", "d3q27.cuh", "philox.cuh", "rflbm_internal.h",
                        "rflbm_step_tma.cu", "rflbm_step_tma16.cu", "step_tma.cuh", "storage.cuh",
                        "tma.cuh")
+FLAT_KERNEL_SOURCES = STEP_KERNEL_SOURCES + ("step_flat.cuh", "rflbm_step_flat.cu", "rflbm_step_flat16.cu",
+                                             "rflbm_step_flat_aa.cu")
 AA_KERNEL_SOURCES = STEP_KERNEL_SOURCES + ("step_aa.cuh", "rflbm_step_aa_f32.cu", "rflbm_step_aa_f16.cu",
                                            "rflbm_step_aa_bf16.cu")
 BATCH_KERNEL_SOURCES = ("collide.cuh", "d3q27.cuh", "philox.cuh", "rflbm_internal.h", "storage.cuh", "tma.cuh",
@@ -169,14 +171,21 @@ def kernel_name(kind, path, kT, model, storage="f32", pattern="pingpong", sites_
 def _kernel_name(kind, path, kT, model, storage, pattern, sites_per_thread, odd_sites_per_thread):
     noise = "noise" if kT > 0 else "no noise"
     m = "BGK" if model else "Reg"
+    flat = kind == 2 and path == 0  # tiles of consecutive sites instead of row segments
     if pattern == "aa":
         if kind == 2:
             odd = sites_per_thread if odd_sites_per_thread is None else odd_sites_per_thread
             even_k = "step_aa_even_pair" if sites_per_thread == 2 else "step_aa_even"
             odd_k = "step_aa_odd_pair" if odd == 2 else "step_aa_odd"
             tag = {(1, 1): "", (2, 2): "pair_", (1, 2): "oddpair_", (2, 1): "evenpair_"}[(sites_per_thread, odd)]
+            if flat:
+                even_k, odd_k = (k.replace("step_aa", "step_flat_aa") for k in (even_k, odd_k))
+                return f"{even_k}+{odd_k}<{storage}, {m}, {noise}>", f"step_flat_aa_{tag}{storage}"
             return f"{even_k}+{odd_k}<{storage}, {path}, {m}, {noise}>", f"step_aa_{tag}{storage}_{path}"
         return f"step_aa_gather<{storage}, {m}, {noise}>", f"step_aa_gather_{storage}"
+    if flat:
+        pair = "_pair" if sites_per_thread == 2 else ""
+        return f"step_flat{pair}<{storage}, {m}, {noise}>", f"step_flat{pair}_{storage}"
     if kind == 2 and sites_per_thread == 2:
         return f"step_tma_pair<{storage}, {path}, {m}, {noise}>", f"step_tma_pair_{storage}_{path}"
     if kind == 2:
@@ -195,6 +204,7 @@ def profiled_traffic(profile_stem, edge):
         return None
     m = re.search(r"traffic_bytes_per_(?:launch|step):\s*([0-9.eE+]+)\s*\(sources ([0-9a-f]+)\)", text)
     names = (AA_KERNEL_SOURCES if profile_stem.startswith("step_aa") else
+             FLAT_KERNEL_SOURCES if profile_stem.startswith("step_flat") else
              BATCH_KERNEL_SOURCES if profile_stem.startswith("k_batch") else STEP_KERNEL_SOURCES)
     if not m or m.group(2) != kernel_source_hash(names):
         return None

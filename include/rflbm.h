@@ -250,13 +250,12 @@ int rflbm_synchronize(rflbm_t* h);
 int rflbm_get_dims(const rflbm_t* h, int* nx, int* ny, int* nz);
 int rflbm_launches_per_step(const rflbm_t* h);
 
-/* Step kernel that the box's rows allow (an rflbm_kernel value other than AUTO): TMA when row
- * segments cover them, and *width, if not NULL, receives the segment width; else the general
- * kernel and 0. (Flat tiles and the general kernel on small boxes, see rflbm_kernel, change neither
- * the report nor the values.) */
+/* Step kernel the handle runs (an rflbm_kernel value other than AUTO). *width, if not NULL, receives
+ * the row-segment width of the TMA kernels, 0 for flat tiles (of 128 sites) and the general kernel: TMA with
+ * width 0 is flat tiles. */
 int rflbm_step_path(const rflbm_t* h, int* width);
 
-/* Sites one thread of the TMA kernel of the next step (rflbm_step(h, 1)) updates: 2 where the
+/* Sites one thread of the kernel of the next step (rflbm_step(h, 1)) updates: 2 where the
  * TMA kernels run their two-site form (packed f32x2 arithmetic, one instruction for both
  * sites): Reg-FLBM with 16-bit storage and float32 without noise in either streaming
  * pattern, and the odd AA steps of float32 Reg-FLBM whose rows span several segments (flat tiles:

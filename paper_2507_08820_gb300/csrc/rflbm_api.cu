@@ -42,14 +42,13 @@ struct rflbm {
   int stat_blocks = 0;
   HostResults* host = nullptr; // page-locked memory that kernels write the results of small calls into
   int* err = nullptr;          // host->err: set by bounded waits in kernels
-  int tma_width = 0;           // row-segment width of the TMA step path (0: generic)
+  int tma_width = 0;           // row-segment width of the TMA step path (0: flat tiles or the general kernel)
   int kernel = RFLBM_KERNEL_GATHER;  // the step kernel in use
   CUtensorMap load_map[2];     // per buffer: source-row loads with halo
   CUtensorMap store_map[2];    // per buffer: row-segment stores
   CUtensorMap row_map;         // AA with one segment per row: three-plane row stores
   uint32_t test_extra_tx = 0;  // testing hook (rflbm_testing_expect_extra_bytes)
   bool has_row_map = false;
-  bool small = false;          // the steps run in the general kernel for their latency
   bool flat = false;           // the steps run in flat tiles (load_map, store_map are then flat)
   // diagnostics (allocated on first use)
   double* diag_partials = nullptr;
@@ -304,14 +303,13 @@ void setup_tma(rflbm* h) {
   h->tma_width = 0;
   h->kernel = RFLBM_KERNEL_GATHER;
   const int st = h->variant.storage;
-  h->small = general_pays(h);
+  if (general_pays(h)) return;
   int w = tma_segment_width(h->geo.nx);
   // rows that no width divides: ragged last segments (whose excess threads store nothing)
   if (w == 0) w = tma_ragged_width(h->geo.nx, storage_bytes(st));
   if (setup_flat(h)) {
     h->flat = true;
-    h->tma_width = w;
-    h->kernel = w ? RFLBM_KERNEL_TMA : RFLBM_KERNEL_GATHER;
+    h->kernel = RFLBM_KERNEL_TMA;
     return;
   }
   if (w == 0 || h->cfg.kernel == RFLBM_KERNEL_GATHER) return;
@@ -636,7 +634,6 @@ cudaError_t launch_rows(rflbm* h, StepParams& p, uint32_t row0, uint32_t nrows, 
   if (h->aa) {
     p.src = p.dst = h->buf[0];
     const bool odd = h->phase != 0;
-    if (h->small) return launch_step_aa_gather(p, h->variant, odd, h->stream);
     if (h->flat) {
       const TmaMaps m{&h->load_map[0], &h->store_map[0], 0};
       return launch_step_flat_aa(m, p, h->variant, odd, h->stream);
@@ -649,7 +646,6 @@ cudaError_t launch_rows(rflbm* h, StepParams& p, uint32_t row0, uint32_t nrows, 
   }
   p.src = h->buf[h->cur];
   p.dst = h->buf[1 - h->cur];
-  if (h->small) return launch_step_gather(p, h->variant, h->stream);
   if (h->flat) {
     const TmaMaps m{&h->load_map[h->cur], &h->store_map[1 - h->cur], 0};
     return launch_step_flat(m, p, h->variant, h->stream);
@@ -1059,7 +1055,7 @@ int rflbm_step_path(const rflbm_t* h, int* width) {
 
 int rflbm_step_sites_per_thread(const rflbm_t* h) {
   if (int e = check_handle(h)) return e;
-  if (h->kernel != RFLBM_KERNEL_TMA && !h->flat) return 1;
+  if (h->kernel != RFLBM_KERNEL_TMA) return 1;
   if (h->flat)
     return (h->aa ? flat_aa_uses_pairs(h->variant, h->phase != 0, h->geo.nx) : tma_uses_pairs(h->variant)) ? 2 : 1;
   if (h->aa) return aa_uses_pairs(h->variant, h->phase != 0, h->has_row_map) ? 2 : 1;

@@ -395,7 +395,7 @@ def rflbm_testing_noise_time(nsites):
 
 
 def rflbm_step_path(h):
-    """(kernel, row-segment width) of the step kernel the handle runs."""
+    """(kernel, row-segment width) of the step kernel the handle runs; TMA with width 0: flat tiles."""
     w = C.c_int()
     k = _check(lib.rflbm_step_path(h, C.byref(w)))
     return k, w.value

@@ -77,3 +77,13 @@ def test_mode_norms_match_the_oracle():
     import numpy as np
     from oracle import rflbm_oracle as o
     assert np.allclose(bench.mode_norms(), o.norms(), rtol=0, atol=1e-15)
+
+
+def test_flat_tiles_are_named_by_the_kernels_that_run():
+    """A step path of TMA without a row-segment width is flat tiles."""
+    assert bench.kernel_name(2, 0, 1e-4, 0) == ("step_flat<f32, Reg, noise>", "step_flat_f32")
+    assert bench.kernel_name(2, 0, 0.0, 0, "f16", "pingpong", 2) == (
+        "step_flat_pair<f16, Reg, no noise>", "step_flat_pair_f16_kt0")
+    assert bench.kernel_name(2, 0, 1e-4, 0, "f32", "aa", 1, 2) == (
+        "step_flat_aa_even+step_flat_aa_odd_pair<f32, Reg, noise>", "step_flat_aa_oddpair_f32")
+    assert set(bench.FLAT_KERNEL_SOURCES) > set(bench.STEP_KERNEL_SOURCES)
