@@ -86,3 +86,33 @@ def test_flat_tiles_report_an_expired_wait(R):
         st, status = R.rflbm_stats(box.h)
         assert status == R.RFLBM_OK and abs(st.mass - box.n) < 1e-5 * box.n
         box.close()
+
+
+# without noise flat tiles start at 450,000 sites in float32 and 230,000 in 16-bit storage: the edge geometries above that
+# line (the shortest rows, one row of a box, one slab of rows, a single row, a last tile of one site, rows of 30 sites)
+STILL_SHAPES = [(16, 121, 240), (17, 113, 240), (131, 1, 3500), (401, 1151, 1), (460033, 1, 1), (30, 160, 96), (100, 50, 91),
+                (1002, 2, 231), (150, 44, 70)]
+
+
+@pytest.mark.parametrize("pattern", [0, 1])
+@pytest.mark.parametrize("kw", [dict(), dict(storage=1), dict(storage=2), dict(model=1), dict(model=1, storage=2),
+                                dict(omega_g=1.3)])
+@pytest.mark.parametrize("shape", STILL_SHAPES)
+def test_flat_tiles_without_noise_match_the_gather_kernel_bitwise(R, shape, kw, pattern):
+    if pattern == 1 and "omega_g" in kw:
+        pytest.skip("AA steps run Reg-FLBM with omega_g = 1, or BGK")
+    kw = dict(kw, kT=0.0, pattern=pattern)
+    box = R.Box(*shape, tau=0.7, **kw)
+    assert R.rflbm_step_path(box.h) == (R.RFLBM_KERNEL_TMA, 0)
+    box.close()
+    _agree(R, shape, kw)
+
+
+@pytest.mark.parametrize("shape", [s for s in SHAPES if s[0] not in (288, 320, 1000)])
+@pytest.mark.parametrize("kw", [kw for kw in VARIANTS if kw["kT"] > 0])
+def test_the_boxes_with_noise_above_run_flat_tiles(R, shape, kw):
+    """What the comparisons with the gather kernel rest on (rows in segments of 64 or 96 sites run flat tiles in some
+    variants only, rows of 1000 ragged segments)."""
+    box = R.Box(*shape, tau=0.7, **kw)
+    assert R.rflbm_step_path(box.h) == (R.RFLBM_KERNEL_TMA, 0)
+    box.close()
