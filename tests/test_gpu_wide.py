@@ -231,3 +231,25 @@ def test_initial_fields_where_a_velocity_term_cancels(R, others):
     stored = (got.astype(np.longdouble) - w).astype(np.float32)  # (the export rounds f to FP64)
     tol = 0.5000001 * np.spacing(np.abs(stored)).astype(float) + 16 * EPS * size
     assert np.all(np.abs(stored.astype(np.longdouble) - (f - w)) <= tol)
+
+
+@pytest.mark.parametrize("unit", [2.0 ** -40, 2.0 ** -22, 2.0 ** 40, 2.0 ** 85])
+def test_velocities_are_fp64_quotients(R, unit):
+    """Populations of whole units, so that the sums are exact in FP64 and so is their conversion: u is then the quotient of
+    the same two numbers, to 2 units in the last place of the correctly rounded one (a reciprocal by Newton steps, a
+    quotient corrected once by its remainder). 2^12 to 2^20 units a population; at 2^85 densities pass 2^107."""
+    g = np.random.default_rng(29)
+    n = 20000
+    k = g.integers(2 ** 12, 2 ** 20, (27, n)) * g.choice([-1, 1], (27, n))
+    k[:, : n // 2] = np.abs(k[:, : n // 2])  # half of the sites with densities far from zero
+    v = k * unit
+    f = o.weights()[:, None] + v  # rounds to FP64; g = f - w rho0 is v again in float32
+    box = R.Box(n, 1, 1, tau=0.8)
+    R.rflbm_set_populations(box.h, np.ascontiguousarray(f))
+    rho, u, _ = box.macroscopic()
+    box.close()
+    wrho = 1.0 + k.sum(axis=0) * unit
+    assert np.array_equal(rho, wrho)
+    j = (o.velocities().T @ k) * unit
+    want = j / wrho
+    assert np.all(np.abs(u - want) <= 2 * np.spacing(np.abs(want)))
