@@ -222,23 +222,21 @@ __global__ void k_get_sites(Geometry g, float rho0, StoreScale ss,
   }
 }
 
-// Raw moments of order <= 2 of the shifted populations of one site, summed in Acc
-// (double for the moments export; float for the global diagnostics, whose values are of
-// order sqrt(kT) because the rest state is subtracted), returned in FP64.
+// Raw moments of order <= 2 of the shifted populations of one site in FP64.
 struct SiteMoments {
   double drho, j[3], s[6];  // s: sum g c_a c_b for xx, yy, zz, xy, xz, yz
 };
 
-template <int kStore, class Acc>
+template <int kStore>
 __device__ __forceinline__ SiteMoments site_moments(const Geometry& g, uint32_t s,
                                                     const typename Storage<kStore>::T* src,
                                                     const StoreScale& ss) {
   const PopSlots slots(s, g);
   using S = Storage<kStore>;
-  Acc drho = 0, j0 = 0, j1 = 0, j2 = 0, s0 = 0, s1 = 0, s2 = 0, s3 = 0, s4 = 0, s5 = 0;
+  double drho = 0, j0 = 0, j1 = 0, j2 = 0, s0 = 0, s1 = 0, s2 = 0, s3 = 0, s4 = 0, s5 = 0;
 #pragma unroll
   for (int i = 0; i < kQ; ++i) {
-    const Acc v = (Acc)S::load(src[slots(i)], class_of(i), ss);
+    const double v = (double)S::load(src[slots(i)], class_of(i), ss);
     const int cx = cx_of(i), cy = cy_of(i), cz = cz_of(i);
     drho += v;
     if (cx) j0 += cx * v;
@@ -263,7 +261,7 @@ template <int kStore>
 __device__ __noinline__ void moments_fp64(const Geometry& g, uint32_t s, const StoreScale& ss,
                                           const typename Storage<kStore>::T* src, double rho0, double* rho, double* u,
                                           double* pi) {
-  const SiteMoments m = site_moments<kStore, double>(g, s, src, ss);
+  const SiteMoments m = site_moments<kStore>(g, s, src, ss);
   const double r = rho0 + m.drho;
   if (rho) rho[s] = r;
   if (u) {

@@ -964,9 +964,8 @@ rflbm_batch_t* rflbm_batch_create(const rflbm_replica_t* reps, int n, double rho
     if (e != cudaSuccess) rc = bcuda(e, "allocating batch descriptors");
   }
   if (rc == RFLBM_OK) {
-    int64_t nmax = 0;
-    for (int r = 0; r < n; ++r) nmax = std::max<int64_t>(nmax, b->host[r].geo.n);
-    b->stat_blocks = std::max(1, (int)std::min<int64_t>(3 * (int64_t)b->num_sms, (nmax + 255) / 256));
+    for (int r = 0; r < n; ++r)
+      b->stat_blocks = std::max(b->stat_blocks, stats_partial_blocks(b->host[r].geo, b->num_sms));
     cudaError_t e = cudaMalloc((void**)&b->partials, sizeof(double) * ((size_t)b->stat_blocks * kStatOutFields + 1));
     if (e == cudaSuccess)
       e = cudaMemset(b->partials + (size_t)b->stat_blocks * kStatOutFields, 0, sizeof(double));
@@ -1085,7 +1084,7 @@ int rflbm_batch_stats(rflbm_batch_t* b, int r, rflbm_stats_t* out) {
   if (!b || r < 0 || r >= b->n || !out) return bfail(RFLBM_EINVAL, "invalid batch, replica or output");
   if (!b->initialised) return bfail(RFLBM_ESTATE, "batch state not initialised");
   const ReplicaDev& d = b->host[r];
-  const int blocks = std::max(1, (int)std::min<int64_t>(b->stat_blocks, ((int64_t)d.geo.n + 255) / 256));
+  const int blocks = stats_partial_blocks(d.geo, b->num_sms);
   const double* const host = b->results->stats;
   unsigned* const done = reinterpret_cast<unsigned*>(b->partials + (size_t)b->stat_blocks * kStatOutFields);
   BCUDA(launch_stats(d.geo, d.cp.rho0, d.ss, b->storage, d.buf[b->cur], b->partials, blocks, b->results->stats, done,

@@ -291,7 +291,7 @@ bool spectrum_axis(int n, SpectrumAxis* ax) {
   if (n < 1 || n > kMaxLine) return false;
   const int radices[8] = {8, 4, 2, 3, 5, 7, 11, 13};
   for (int r : radices)
-    while (n % r == 0 && !(r == 4 && n % 8 == 0)) {
+    while (n % r == 0) {
       if (r == 3 || r == 5 || r == 7) ax->odd = ax->odd > 1 ? ax->odd : 1;
       if (r > 8) ax->odd = 2;
       ax->factors[ax->nfactors++] = r;

@@ -9,12 +9,13 @@
 // its own site of the other buffer (27 coalesced stores).
 // Algorithmic traffic per site update: 27 populations read + 27 written (216 bytes in
 // float32, 108 bytes in 16-bit storage).
-// On large boxes the TMA kernels are faster. On small ones, whose grid is resident at once, a step
-// lasts as long as its chain of launch, wait, loads, collision and stores, and plain loads and
-// stores make the shortest one. Microseconds per step of 16^3 / 32^3 / 48^3, float32 with noise: 6.2 /
-// 6.2 / 8.2 launched after the previous step had ended, 2.6 / 7.6 / 8.0 with dependent launch
-// and the draw behind the wait, 2.0 / 4.3 / 5.1 as it is; the row-segment TMA kernel takes 6.5 at
-// 32^3. Blocks of 64 threads spread a small box over the SMs (of 256: 2.4 / 4.4 / 5.2).
+// On large boxes the TMA kernels are faster. On small ones a step lasts as long as its chain of
+// launch, wait, loads, collision and stores, and plain loads and stores make the shortest one (general_pays has the
+// sizes where the sides cross, as measured on the 152 SMs of a GB300). Microseconds per step of 16^3 / 32^3 / 48^3,
+// float32 with noise: 6.2 / 6.2 / 8.2 launched after the previous step had ended, 2.6 / 7.6 / 8.0 with
+// dependent launch and the draw behind the wait, 2.0 / 4.3 / 5.1 with the draw ahead of it, 2.2 / 3.6 / 4.8 with the
+// addresses ahead of it too; the row-segment TMA kernel takes 6.5 at 32^3. Blocks of 64 threads spread a small
+// box over the SMs (of 256: 2.4 / 4.4 / 5.2).
 #include "rflbm_internal.h"
 #include "tma.cuh"
 
