@@ -65,12 +65,12 @@ __device__ __noinline__ void init_site_fp64(const Geometry& g, uint32_t s, float
 // The same for every site, scattered to the view's slots. With psi(c, u) = w_c (1 + delta_c),
 // g_i / w_i = Q_ab + (rho0 + Q_ab) delta_c where Q_ab = r D_ab + (r - rho0) and 1 + D_ab =
 // (1 + delta_a)(1 + delta_b): the rest value is no difference any more, so sums of two float32 values
-// carry it to 2^-43 of the magnitudes of its terms, and FP64 differs from it by no more than its own dozen
+// carry it to some 2^-43 of the magnitudes of its terms, and FP64 differs from it by no more than its own dozen
 // roundings of f_i. Where every value within these errors rounds to one float32 value, that is
 // the FP64 result; a site with any population that they leave open is redone in FP64 (one site in
 // thousands for flows with velocities of a percent; most below 1e-6, where g_i is lost in the roundings of
 // f_i, and a warp with one such site takes as long as one of them). Bound by the 32 bytes read and
-// 108 written per site (146 us at 192^3): 192^3 takes 346 us with velocities of 2 %, 1228 us at rest or with
+// 108 written per site (146 us at 192^3): 192^3 takes 367 us with velocities of 2 %, 1229 us at rest or with
 // velocities up to 1e-4, and took 1255 us with 100 FP64 operations for every site.
 template <int kStore>
 __global__ void __launch_bounds__(kAuxBlock) k_init_field(Geometry g, float rho0, StoreScale ss, const double* __restrict__ rho,
@@ -92,6 +92,10 @@ __global__ void __launch_bounds__(kAuxBlock) k_init_field(Geometry g, float rho0
     psi_excess(pair_of(uy), dy, ty);
     psi_excess(pair_of(uz), dz, tz);
     const float own = fmaf(0x1p-43f, fabsf(dR.hi), 0x1p-48f * (fabsf(R.hi) + rho0));
+    // The pairs' errors over R A, A the terms of f_i / w_i r - 1: at most 0.42, 0.67, 1.1, 1.9 and 4.3 times 2^-43 for
+    // velocities of 0.03, 0.1, 0.3, 1 and 10 to 2^16 (the largest of 2 M random sites each); FP64's: below 2^-47.
+    const float corner = fmaf(1.0f + tx[0], fmaf(ty[0], 1.0f + tz[0], tz[0]), tx[0]);  // the largest A of the site
+    const float slope = fmaf(fminf(corner, 8.0f), 0x1p-43f, 0x1.1p-43f);
 #pragma unroll
     for (int a = 0; a < 3; ++a)
 #pragma unroll
@@ -108,7 +112,7 @@ __global__ void __launch_bounds__(kAuxBlock) k_init_field(Geometry g, float rho0
           const Pair32 W{(float)w[cls], (float)(w[cls] - (double)(float)w[cls])};
           const Pair32 v = pmul(W, padd(Q, pmul(P, dz[c])));
           const float A = fmaf(tz[c], 1.0f + Aab, Aab);  // over the terms of f_i / w_i r - 1
-          const float err = W.hi * fmaf(fabsf(R.hi) * A, 0x1.1p-43f, own);
+          const float err = W.hi * fmaf(fabsf(R.hi) * A, slope, own);
           const float lo = __fadd_rn(v.hi, __fsub_rn(v.lo, err));
           open = open || !(lo == __fadd_rn(v.hi, __fadd_rn(v.lo, err)));
           dst[slots(pop_at(a, b, c))] = S::store(lo, cls, ss);

@@ -253,3 +253,30 @@ def test_velocities_are_fp64_quotients(R, unit):
     j = (o.velocities().T @ k) * unit
     want = j / wrho
     assert np.all(np.abs(u - want) <= 2 * np.spacing(np.abs(want)))
+
+
+@pytest.mark.parametrize("rho0,rho,u", [
+    (1.0, 1.0, (-666.7065315539121, 335.5127149724657, 134.1717761152097)),
+    (0.37, float(np.float32(0.37)), (396.84542754641285, -256.2102318772882, -36.53873304552258)),
+    (0.37, float(np.float32(0.37)), (-451.7177706589363, 575.1681675438398, 132.75070061364414)),
+    (2.5, 2.5132507072454056, (791.9933978206979, 236.0201251622538, 757.5623402964293)),
+    (1e-3, 0.0009941081360488576, (30.00013269037117, -29.999999852552524, 29.999999999686505)),
+])
+def test_initial_fields_at_large_velocities(R, rho0, rho, u):
+    """Sites with a population so near the middle of two float32 values that the error of a form in float32 pairs, larger
+    here than for flows, decides between them: the FP64 form rounds to the nearer one, up to its own
+    roundings (as in test_initial_fields_where_a_velocity_term_cancels)."""
+    box = R.Box(1, 1, 1, tau=0.8, rho0=rho0)
+    R.rflbm_init_field(box.h, np.array([rho]), np.array(u)[:, None].copy())
+    got = box.populations()[:, 0]
+    box.close()
+    rho0 = float(np.float32(rho0))
+    w = o.weights().astype(np.longdouble)
+    f, size = w * rho, w * rho
+    for a, c in enumerate(o.velocities().T):
+        v = np.longdouble(u[a])
+        f = f * np.where(c == 0, 1 - 1.5 * v ** 2, 1 + 3 * c * v + 3 * v ** 2)
+        size = size * (1 + 3 * abs(v) + 3 * v ** 2)
+    stored = (got.astype(np.longdouble) - w * rho0).astype(np.float32)  # (the export rounds f to FP64)
+    tol = 0.5000001 * np.spacing(np.abs(stored)).astype(float) + 16 * EPS * size
+    assert np.all(np.abs(stored.astype(np.longdouble) - (f - w * rho0)) <= tol)
