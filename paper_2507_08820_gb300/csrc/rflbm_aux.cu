@@ -11,9 +11,11 @@ constexpr int kAuxBlock = 256;
 __device__ __forceinline__ uint32_t site_of(int64_t t) { return (uint32_t)t; }
 
 // One 1-D factor of the product-form equilibrium (Eq. 26 factorised over the axes):
-// Psi(0, u) = 2/3 - u^2, Psi(+-1, u) = (1/3 +- u + u^2)/2.
+// Psi(0, u) = 2/3 - u^2, Psi(+-1, u) = (1/3 +- u + u^2)/2. Every rounding is spelled out, so that a stored state does
+// not depend on which products a compiler joins with a sum.
 __device__ __forceinline__ double psi(int c, double u) {
-  return c == 0 ? (2.0 / 3.0 - u * u) : 0.5 * (1.0 / 3.0 + c * u + u * u);
+  const double q = __dmul_rn(u, u);
+  return c == 0 ? __dsub_rn(2.0 / 3.0, q) : __dmul_rn(0.5, __dadd_rn(__dadd_rn(1.0 / 3.0, c * u), q));
 }
 
 // Population with the velocity of tile entry (a, b, c) = (c_x + 1, c_y + 1, c_z + 1).
@@ -57,8 +59,9 @@ __device__ __noinline__ void init_site_fp64(const Geometry& g, uint32_t s, float
   const PopSlots slots(s, g);
 #pragma unroll
   for (int i = 0; i < kQ; ++i) {
-    const double f = r * psi(cx_of(i), ux) * psi(cy_of(i), uy) * psi(cz_of(i), uz);
-    dst[slots(i)] = S::store((float)(f - weight_of(i) * (double)rho0), class_of(i), ss);
+    const double f = __dmul_rn(__dmul_rn(r, psi(cx_of(i), ux)), psi(cy_of(i), uy));
+    const double g_i = __fma_rn(f, psi(cz_of(i), uz), -__dmul_rn(weight_of(i), (double)rho0));
+    dst[slots(i)] = S::store((float)g_i, class_of(i), ss);
   }
 }
 
@@ -70,7 +73,7 @@ __device__ __noinline__ void init_site_fp64(const Geometry& g, uint32_t s, float
 // the FP64 result; a site with any population that they leave open is redone in FP64 (one site in
 // thousands for flows with velocities of a percent; most below 1e-6, where g_i is lost in the roundings of
 // f_i, and a warp with one such site takes as long as one of them). Bound by the 32 bytes read and
-// 108 written per site (146 us at 192^3): 192^3 takes 367 us with velocities of 2 %, 1229 us at rest or with
+// 108 written per site (146 us at 192^3): 192^3 takes 367 us with velocities of 2 %, 1270 us at rest or with
 // velocities up to 1e-4, and took 1255 us with 100 FP64 operations for every site.
 template <int kStore>
 __global__ void __launch_bounds__(kAuxBlock) k_init_field(Geometry g, float rho0, StoreScale ss, const double* __restrict__ rho,

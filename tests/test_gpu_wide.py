@@ -280,3 +280,31 @@ def test_initial_fields_at_large_velocities(R, rho0, rho, u):
     stored = (got.astype(np.longdouble) - w * rho0).astype(np.float32)  # (the export rounds f to FP64)
     tol = 0.5000001 * np.spacing(np.abs(stored)).astype(float) + 16 * EPS * size
     assert np.all(np.abs(stored.astype(np.longdouble) - (f - w * rho0)) <= tol)
+
+
+@pytest.mark.parametrize("rho0", [1.0, 0.37])
+@pytest.mark.parametrize("kind", ["rest", "slow", "near one"])
+def test_initial_fields_store_the_spelled_out_fp64_form(R, kind, rho0):
+    """Where the pair form leaves sites open, the stored value is the FP64 form's with the roundings that the kernel spells
+    out: r psi_x psi_y in turn, then one rounding of its product with psi_z less w rho0 (exact fractions here)."""
+    from fractions import Fraction
+    g = np.random.default_rng(31)
+    n, rho0 = 300, float(np.float32(rho0))
+    sign = lambda: g.choice([-1.0, 1.0], (3, n))  # noqa: E731
+    u = {"rest": np.zeros((3, n)), "slow": sign() * 10.0 ** g.uniform(-9, -6, (3, n)),
+         "near one": np.concatenate([sign()[:1] * (1.0 + sign()[:1] * 2.0 ** -g.uniform(20, 30, (1, n))), np.zeros((2, n))])}[kind]
+    rho = rho0 * (1.0 + 1e-9 * g.integers(-1, 2, n))
+    box = R.Box(n, 1, 1, tau=0.8, rho0=rho0)
+    R.rflbm_init_field(box.h, rho, np.ascontiguousarray(u))
+    got = box.populations()
+    box.close()
+    w1 = {0: 2.0 / 3.0, 1: 1.0 / 6.0, -1: 1.0 / 6.0}
+    psi = [{c: 2.0 / 3.0 - v * v if c == 0 else 0.5 * ((1.0 / 3.0 + c * v) + v * v) for c in (-1, 0, 1)} for v in u]
+    want = np.empty((27, n))
+    for i, (cx, cy, cz) in enumerate(o.velocities().tolist()):
+        w = w1[cx] * w1[cy] * w1[cz]
+        f = (rho * psi[0][cx]) * psi[1][cy]
+        for s in range(n):
+            x = Fraction(f[s]) * Fraction(psi[2][cz][s]) - Fraction(w * rho0)
+            want[i, s] = float(np.float32(x.numerator / x.denominator)) + w * rho0  # (as the export returns it)
+    assert np.array_equal(got, want)
