@@ -7,9 +7,9 @@ namespace rflbm_dev {
 // Whole boxes that run in flat tiles. Microseconds per step, float32 with noise unless said, "rows"
 // the row-segment kernels, "ragged" those with a ragged last segment, "gather" the general kernel:
 //  - rows that no segment width divides, from the size where the tiles' longer latency is hidden
-//    (56^3: flat 8.8, gather 8.5; without noise 72^3 12.9 and 11.2, 80^3 15.1 and 15.8; 16-bit without
-//    noise 60^3 8.3 and 7.9, 66^3 8.6 and 9.6): 100^3 flat 38.0, ragged 42.7, gather 49.6, float16
-//    39.7, -, 51.9; 200^3 269, 326, 353, float16 272, 537, 383; 150x110x70 42.9, -, 57.0. Ragged segments
+//    (56^3: flat 8.8, gather 7.6; without noise 72^3 12.9 and 9.7, 80^3 15.0 and 15.7; 16-bit without
+//    noise 60^3 8.3 and 7.5, 66^3 8.6 and 9.0): 100^3 flat 38.0, ragged 42.7, gather 42.3, float16
+//    39.7, -, 43.8; 200^3 269, 326, 316, float16 272, 537, 340; 150x110x70 42.9, -, 48.3. Ragged segments
 //    stay where they are wide and nearly full (376x128x64 102.9 against 103.6, 248x128x64 69.7 and 69.9, AA
 //    75.3 and 76.0; 232x128x64, 10 % idle threads, 69.1 and 65.7), wide with 16-bit storage without
 //    noise (120x128x128 34.5 against 36.8), and for smaller fluctuating ping-pong boxes (60^3: ragged 9.7,
